@@ -25,7 +25,7 @@ struct Tile {
 // (FP64 lattices one cell thick in z with u_z = 0); the host sorts the tiles by
 // constraint system and launches one instantiation for each.
 template <class P, int BLK, bool D2>
-__global__ void __launch_bounds__(BLK) k_batch_step(const BatchEntry* __restrict__ E,
+__global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, 0>)) k_batch_step(const BatchEntry* __restrict__ E,
                                                     const Tile* __restrict__ tiles, int s) {
   extern __shared__ double smem[];
   __shared__ unsigned int s_ctr[CTR_N];
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(BLK) k_batch_step(const BatchEntry* __restrict
     sd.t = st;
   }
   for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
-  load_exp_table();  // also publishes sd and st
+  load_solver_table<in_fixed_point<P, 0>>();  // also publishes sd and st
   const long long t = st;
   if (t < 0) return;  // this lattice has reached its end time (uniform over the block)
   const long long cell = tl.cell0 + threadIdx.x;

@@ -33,7 +33,8 @@ using WS = WSV<double, BLK>;
 constexpr int WS_E = 0;         // normalised equilibrium F_i (39)
 constexpr int WS_LAM = 39;      // multipliers (13)
 constexpr int WS_M = 52;        // normalised targets (13)
-constexpr int WS_DL = 65;       // Newton direction (13)
+constexpr int WS_DL = 65;       // Newton direction (13): only the kernels that solve in FP64
+constexpr int WS_DOUBLES_FX = 65;  // workspace of the kernels that solve in fixed point
 constexpr int WS_DOUBLES = 78;
 
 // Lattice-wide constants of one run.
@@ -44,6 +45,8 @@ struct Phys {
   double tol;       // Newton tolerance on max_k |G_k| / rho
   int maxit;        // Newton updates allowed
   int min_upd;      // updates taken even from a converged warm start
+  unsigned long long tol_fx, tol_fx100;  // tol and tol/100 in units 2^-58 (the fixed-point solve)
+  int fx;           // the fixed-point solve resolves tol (else every solve is FP64)
   int kn_sensor;    // Eq. (alpha) on/off
   double omega[4];  // 1 / (tau alpha) for the four branches of Eq. (alpha) (1/tau without
                     // the sensor), formed on the host with IEEE division
@@ -55,9 +58,13 @@ struct Phys {
 // rcp32: the PTX instruction rcp.approx.ftz.f32 (at most 1 ulp, i.e. relative
 // error <= 2^-23, subnormals flushed to zero).
 __device__ __forceinline__ float rcp32(float x) {
+#ifdef __CUDACC__
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+#else  // the host build of this arithmetic (tests)
+  return 1.0f / x;
+#endif
 }
 
 // rcp64: 1/d for normal d by Newton's method for the root of 1/r - d,
@@ -65,8 +72,12 @@ __device__ __forceinline__ float rcp32(float x) {
 // the hardware estimate rcp.approx.ftz.f64.  Within 2 ulp of 1/d (tested
 // against CUDA's division through lbm39_selftest_rcp).
 __device__ __forceinline__ double rcp64(double d) {
+#ifdef __CUDACC__
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+#else
+  double r = 1.0f / (float)d;
+#endif
   r = fma(r, fma(-d, r, 1.0), r);
   return fma(r, fma(-d, r, 1.0), r);
 }
@@ -131,10 +142,10 @@ __device__ __noinline__ void exp_all_slow(double* Fp) {
 // from_F: F already holds exp(Phi lam) (kept from the previous step), so only
 // the moments are formed -- the same numbers, bit for bit, as evaluating again.
 // D2: z-mirrored velocities share their exponential.
-template <int BLK, bool D2 = false>
-__device__ __forceinline__ void eval_equilibrium(WS<BLK> lam, WS<BLK> dl, double t, WS<BLK> F,
+template <int BLK, bool D2 = false, class DL>
+__device__ __forceinline__ void eval_equilibrium(WS<BLK> lam, DL dl, double t, WS<BLK> F,
                                                  WS<BLK> m, double (&G)[Sys<D2>::N],
-                                                 bool from_F) {
+                                                 bool from_F, const double* __restrict__ tab) {
   using S = Sys<D2>;
   if (!from_F) {
     double l[NM], x[Q];
@@ -160,7 +171,7 @@ __device__ __forceinline__ void eval_equilibrium(WS<BLK> lam, WS<BLK> dl, double
       // per z-mirror pair, then copied
 #pragma unroll 1
       for (int i = 0; i < Q; ++i)
-        if (!D2 || ((kZOwn >> i) & 1ull)) F[i] = exp_tang_core(F[i]);
+        if (!D2 || ((kZOwn >> i) & 1ull)) F[i] = exp_tang_core(F[i], tab);
       if constexpr (D2) {
         static_for<0, Q>([&](auto I) {
           constexpr int i = decltype(I)::value;
@@ -329,8 +340,8 @@ __device__ __noinline__ bool dir32(const float* __restrict__ Fp, float* __restri
 // b and delta in dl.  FP64 path: J and LDL^T in FP64.  Precision form: in
 // FP32 (dir32; the residual and the update stay FP64, so the iteration still
 // converges to the FP64 root).
-template <int BLK, bool MIXED, bool D2 = false>
-__device__ __forceinline__ bool newton_direction(WS<BLK> F, WS<BLK> dl) {
+template <int BLK, bool MIXED, bool D2 = false, class DL>
+__device__ __forceinline__ bool newton_direction(WS<BLK> F, DL dl) {
   constexpr int N = Sys<D2>::N;
   if constexpr (!MIXED) {
     double J[N * (N + 1) / 2], s[N], b[N], rd[N];
@@ -392,16 +403,19 @@ struct NewtonResult {
 // cached: F already holds exp(Phi lam) for the starting lam (the previous
 // step's last evaluation, kept per cell), so the first evaluation skips the
 // exponentials.
-template <int BLK, bool MIXED, bool D2 = false>
-__device__ NewtonResult newton(WS<BLK> w, const Phys& ph, int maxit, bool cached) {
+// In FP64 throughout (MIXED: but for the direction); dl: where the direction is kept; tab: the
+// exponential's table.
+template <int BLK, bool MIXED, bool D2, class DL>
+__device__ __forceinline__ NewtonResult newton_in(WS<BLK> w, DL dl, const double* tab, double tol,
+                                                  int min_upd, int maxit, bool cached) {
   using S = Sys<D2>;
-  WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M), dl = w.at(WS_DL);
+  WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M);
   int n = 0, failed = 0, ls = 0;
   bool first = true, polished = false, restore = false;
   double t = 0.0, s0 = 0.0;  // trial point lam - t dl
   for (;;) {
     double G[S::N];
-    eval_equilibrium<BLK, D2>(lam, dl, t, F, m, G, first && cached);
+    eval_equilibrium<BLK, D2>(lam, dl, t, F, m, G, first && cached, tab);
     if (restore) break;  // F is back at the last accepted lam after a failed line search
     if (!first && !polished && !(sum_sq(G) < s0)) {  // reject: halve the step
       if (++ls > LS_MAX) {
@@ -421,17 +435,26 @@ __device__ NewtonResult newton(WS<BLK> w, const Phys& ph, int maxit, bool cached
     if (!first) ++n;
     first = false;
     const double r = max_abs(G);
-    if (n >= ph.min_upd && r < ph.tol && (r < 1e-2 * ph.tol || polished)) break;
+    if (n >= min_upd && r < tol && (r < 1e-2 * tol || polished)) break;
     if (n >= maxit) { failed = 1; break; }
     s0 = sum_sq(G);
 #pragma unroll
     for (int k = 0; k < S::N; ++k) dl[k] = G[k];
     if (!newton_direction<BLK, MIXED, D2>(F, dl)) { failed = 1; break; }
-    polished = r < ph.tol;
+    polished = r < tol;
     t = 1.0;
     ls = 0;
   }
   return NewtonResult{n, failed};
+}
+
+// The solve of the cells outside the ranges of newton_fx, and of single states: not inlined, as
+// few cells take it, its direction on the stack.
+template <int BLK, bool MIXED, bool D2 = false>
+__device__ __noinline__ NewtonResult newton(WS<BLK> w, double tol, int min_upd, int maxit,
+                                            bool cached) {
+  double dlv[Sys<D2>::N];
+  return newton_in<BLK, MIXED, D2>(w, WS<1>{dlv}, gen::kExp2Table, tol, min_upd, maxit, cached);
 }
 
 // Single-precision start of a solve (root finder 3, and the precision form's
@@ -529,7 +552,7 @@ __device__ NewtonResult newton_chord(WS<BLK> w, const Phys& ph, int maxit, bool 
   double Jf[N * (N + 1) / 2], rd[N];
   for (;;) {
     double G[N];
-    eval_equilibrium<BLK, D2>(lam, dl, t, F, m, G, first && cached);
+    eval_equilibrium<BLK, D2>(lam, dl, t, F, m, G, first && cached, exp_table());
     if (restore) break;  // F is back at the last accepted lam after a failed line search
     if (refresh) {
       refresh = false;  // back at lam after a rejected chord step: a Newton step from here
@@ -626,7 +649,7 @@ constexpr int RETRY_PERIOD = 8;  // a power of two
 // phi_k(xi_i) at that point, and G = sum_i F_i phi5(xi_i) - m5 (phi5 = [1, xi,
 // |xi|^2], so its sums are s_0..s_3 and s_4 + s_5 + s_6).
 template <int BLK>
-__device__ __forceinline__ void eval5(WS<BLK> mu, WS<BLK> dl, double t, WS<BLK> F,
+__device__ __forceinline__ void eval5(WS<BLK> mu, WS<1> dl, double t, WS<BLK> F,
                                       const double (&m5)[N5], double (&G)[N5],
                                       double (&s)[NM]) {
   double v[N5];
@@ -647,7 +670,7 @@ __device__ __forceinline__ void eval5(WS<BLK> mu, WS<BLK> dl, double t, WS<BLK> 
   } else {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      x[i] = exp_tang_core(x[i]);
+      x[i] = exp_tang_core(x[i], gen::kExp2Table);
       F[i] = x[i];
     }
   }
@@ -717,11 +740,12 @@ __device__ __forceinline__ bool is_fallback_embedding(WS<BLK> lam) {
 // The fallback equilibrium into F for the cell whose 13 normalised targets
 // are in the workspace (m: their u and second moments give the five targets),
 // from the five multipliers warm[] (a stored embedding) or, with warm null, the
-// Gaussian start; leaves mu in the first five m slots and overwrites the dl
-// slots.  Returns 1 if its solve fails too (F then holds a partial iterate).
+// Gaussian start; leaves mu in the first five m slots.  Returns 1 if its solve fails too (F then holds a partial iterate).
 template <int BLK>
 __device__ __noinline__ int fallback_equilibrium(WS<BLK> w, double T, const double* warm) {
-  WS<BLK> F = w.at(WS_E), mu = w.at(WS_M), dl = w.at(WS_DL);
+  WS<BLK> F = w.at(WS_E), mu = w.at(WS_M);
+  double dlv[N5];
+  const WS<1> dl{dlv};
   const double m5[N5] = {1.0, mu[1], mu[2], mu[3], mu[4] + mu[5] + mu[6]};
   double G[N5], s[NM];
   if (warm) {

@@ -1045,7 +1045,7 @@ constexpr double EXP_INV_L = 369.3299304675746;
 constexpr double EXP_L_HI = 0.0027076061742263846;
 constexpr double EXP_L_LO = -1.6409824502660487e-13;
 // 2^(j/256), j = 0..255, each the double nearest the exact value.
-__device__ __constant__ double kExp2Table[256] = {
+__device__ const double kExp2Table[256] = {
     1.0, 1.0027112750502025, 1.0054299011128027, 1.0081558981184175,
     1.0108892860517005, 1.0136300849514894, 1.016378314910953, 1.019133996077738,
     1.0218971486541166, 1.0246677928971357, 1.0274459491187637, 1.030231637686041,
@@ -1110,6 +1110,1048 @@ __device__ __constant__ double kExp2Table[256] = {
     1.9360617934922943, 1.9413109895286405, 1.9465744175792332, 1.9518521162309783,
     1.9571441241754002, 1.9624504802089273, 1.9677712232331759, 1.9731063922552343,
     1.978456026387951, 1.9838201648502194, 1.9891988469672663, 1.9945921121709402,
+};
+
+// A velocity index as a type.
+template <int I>
+struct Idx {
+  static constexpr int value = I;
+};
+
+// s_k = sum_i v(i) phi_k(xi_i) in 64-bit integers.
+template <class V>
+__device__ __forceinline__ void sums_fx(const V& v, unsigned long long (&s)[13]) {
+  const unsigned long long v0 = v(Idx<0>{});
+  s[0] = v0;
+  const unsigned long long v5 = v(Idx<5>{});
+  const unsigned long long v6 = v(Idx<6>{});
+  const unsigned long long w1_0_0 = v5 + v6;
+  const unsigned long long w1_0_1 = v5 - v6;
+  s[0] += w1_0_0;
+  s[6] = w1_0_0;
+  s[3] = w1_0_1;
+  s[12] = w1_0_1;
+  const unsigned long long v19 = v(Idx<19>{});
+  const unsigned long long v20 = v(Idx<20>{});
+  const unsigned long long w2_0_0 = v19 + v20;
+  const unsigned long long w2_0_1 = v19 - v20;
+  s[0] += w2_0_0;
+  s[6] += 4ull * w2_0_0;
+  s[3] += 2ull * w2_0_1;
+  s[12] += 8ull * w2_0_1;
+  const unsigned long long v37 = v(Idx<37>{});
+  const unsigned long long v38 = v(Idx<38>{});
+  const unsigned long long w3_0_0 = v37 + v38;
+  const unsigned long long w3_0_1 = v37 - v38;
+  s[0] += w3_0_0;
+  s[6] += 9ull * w3_0_0;
+  s[3] += 3ull * w3_0_1;
+  s[12] += 27ull * w3_0_1;
+  const unsigned long long v3 = v(Idx<3>{});
+  const unsigned long long v4 = v(Idx<4>{});
+  const unsigned long long w4_0_0 = v3 + v4;
+  const unsigned long long w4_0_1 = v3 - v4;
+  s[0] += w4_0_0;
+  s[5] = w4_0_0;
+  s[2] = w4_0_1;
+  s[11] = w4_0_1;
+  const unsigned long long v17 = v(Idx<17>{});
+  const unsigned long long v18 = v(Idx<18>{});
+  const unsigned long long w5_0_0 = v17 + v18;
+  const unsigned long long w5_0_1 = v17 - v18;
+  s[0] += w5_0_0;
+  s[5] += 4ull * w5_0_0;
+  s[2] += 2ull * w5_0_1;
+  s[11] += 8ull * w5_0_1;
+  const unsigned long long v29 = v(Idx<29>{});
+  const unsigned long long v30 = v(Idx<30>{});
+  const unsigned long long v31 = v(Idx<31>{});
+  const unsigned long long v32 = v(Idx<32>{});
+  const unsigned long long w6_0_0 = v31 + v30;
+  const unsigned long long w6_0_1 = v31 - v30;
+  const unsigned long long w6_0_2 = v29 + v32;
+  const unsigned long long w6_0_3 = v29 - v32;
+  const unsigned long long w6_1_0 = w6_0_2 + w6_0_0;
+  const unsigned long long w6_1_1 = w6_0_2 - w6_0_0;
+  const unsigned long long w6_1_2 = w6_0_3 + w6_0_1;
+  const unsigned long long w6_1_3 = w6_0_3 - w6_0_1;
+  s[0] += w6_1_0;
+  s[5] += 4ull * w6_1_0;
+  s[6] += 4ull * w6_1_0;
+  s[3] += 2ull * w6_1_1;
+  s[12] += 16ull * w6_1_1;
+  s[2] += 2ull * w6_1_2;
+  s[11] += 16ull * w6_1_2;
+  s[9] = 4ull * w6_1_3;
+  const unsigned long long v35 = v(Idx<35>{});
+  const unsigned long long v36 = v(Idx<36>{});
+  const unsigned long long w7_0_0 = v35 + v36;
+  const unsigned long long w7_0_1 = v35 - v36;
+  s[0] += w7_0_0;
+  s[5] += 9ull * w7_0_0;
+  s[2] += 3ull * w7_0_1;
+  s[11] += 27ull * w7_0_1;
+  const unsigned long long v1 = v(Idx<1>{});
+  const unsigned long long v2 = v(Idx<2>{});
+  const unsigned long long w8_0_0 = v1 + v2;
+  const unsigned long long w8_0_1 = v1 - v2;
+  s[0] += w8_0_0;
+  s[4] = w8_0_0;
+  s[1] = w8_0_1;
+  s[10] = w8_0_1;
+  const unsigned long long v7 = v(Idx<7>{});
+  const unsigned long long v8 = v(Idx<8>{});
+  const unsigned long long v9 = v(Idx<9>{});
+  const unsigned long long v10 = v(Idx<10>{});
+  const unsigned long long v11 = v(Idx<11>{});
+  const unsigned long long v12 = v(Idx<12>{});
+  const unsigned long long v13 = v(Idx<13>{});
+  const unsigned long long v14 = v(Idx<14>{});
+  const unsigned long long w9_0_0 = v14 + v8;
+  const unsigned long long w9_0_1 = v14 - v8;
+  const unsigned long long w9_0_2 = v11 + v10;
+  const unsigned long long w9_0_3 = v11 - v10;
+  const unsigned long long w9_0_4 = v9 + v12;
+  const unsigned long long w9_0_5 = v9 - v12;
+  const unsigned long long w9_0_6 = v7 + v13;
+  const unsigned long long w9_0_7 = v7 - v13;
+  const unsigned long long w9_1_0 = w9_0_4 + w9_0_0;
+  const unsigned long long w9_1_1 = w9_0_4 - w9_0_0;
+  const unsigned long long w9_1_2 = w9_0_6 + w9_0_2;
+  const unsigned long long w9_1_3 = w9_0_6 - w9_0_2;
+  const unsigned long long w9_1_4 = w9_0_5 + w9_0_1;
+  const unsigned long long w9_1_5 = w9_0_5 - w9_0_1;
+  const unsigned long long w9_1_6 = w9_0_7 + w9_0_3;
+  const unsigned long long w9_1_7 = w9_0_7 - w9_0_3;
+  const unsigned long long w9_2_0 = w9_1_2 + w9_1_0;
+  const unsigned long long w9_2_1 = w9_1_2 - w9_1_0;
+  const unsigned long long w9_2_2 = w9_1_3 + w9_1_1;
+  const unsigned long long w9_2_3 = w9_1_3 - w9_1_1;
+  const unsigned long long w9_2_4 = w9_1_6 + w9_1_4;
+  const unsigned long long w9_2_5 = w9_1_6 - w9_1_4;
+  const unsigned long long w9_2_6 = w9_1_7 + w9_1_5;
+  const unsigned long long w9_2_7 = w9_1_7 - w9_1_5;
+  s[0] += w9_2_0;
+  s[4] += w9_2_0;
+  s[5] += w9_2_0;
+  s[6] += w9_2_0;
+  s[3] += w9_2_1;
+  s[12] += 3ull * w9_2_1;
+  s[2] += w9_2_2;
+  s[11] += 3ull * w9_2_2;
+  s[9] += w9_2_3;
+  s[1] += w9_2_4;
+  s[10] += 3ull * w9_2_4;
+  s[8] = w9_2_5;
+  s[7] = w9_2_6;
+  const unsigned long long v15 = v(Idx<15>{});
+  const unsigned long long v16 = v(Idx<16>{});
+  const unsigned long long w10_0_0 = v15 + v16;
+  const unsigned long long w10_0_1 = v15 - v16;
+  s[0] += w10_0_0;
+  s[4] += 4ull * w10_0_0;
+  s[1] += 2ull * w10_0_1;
+  s[10] += 8ull * w10_0_1;
+  const unsigned long long v25 = v(Idx<25>{});
+  const unsigned long long v26 = v(Idx<26>{});
+  const unsigned long long v27 = v(Idx<27>{});
+  const unsigned long long v28 = v(Idx<28>{});
+  const unsigned long long w11_0_0 = v27 + v26;
+  const unsigned long long w11_0_1 = v27 - v26;
+  const unsigned long long w11_0_2 = v25 + v28;
+  const unsigned long long w11_0_3 = v25 - v28;
+  const unsigned long long w11_1_0 = w11_0_2 + w11_0_0;
+  const unsigned long long w11_1_1 = w11_0_2 - w11_0_0;
+  const unsigned long long w11_1_2 = w11_0_3 + w11_0_1;
+  const unsigned long long w11_1_3 = w11_0_3 - w11_0_1;
+  s[0] += w11_1_0;
+  s[4] += 4ull * w11_1_0;
+  s[6] += 4ull * w11_1_0;
+  s[3] += 2ull * w11_1_1;
+  s[12] += 16ull * w11_1_1;
+  s[1] += 2ull * w11_1_2;
+  s[10] += 16ull * w11_1_2;
+  s[8] += 4ull * w11_1_3;
+  const unsigned long long v21 = v(Idx<21>{});
+  const unsigned long long v22 = v(Idx<22>{});
+  const unsigned long long v23 = v(Idx<23>{});
+  const unsigned long long v24 = v(Idx<24>{});
+  const unsigned long long w12_0_0 = v23 + v22;
+  const unsigned long long w12_0_1 = v23 - v22;
+  const unsigned long long w12_0_2 = v21 + v24;
+  const unsigned long long w12_0_3 = v21 - v24;
+  const unsigned long long w12_1_0 = w12_0_2 + w12_0_0;
+  const unsigned long long w12_1_1 = w12_0_2 - w12_0_0;
+  const unsigned long long w12_1_2 = w12_0_3 + w12_0_1;
+  const unsigned long long w12_1_3 = w12_0_3 - w12_0_1;
+  s[0] += w12_1_0;
+  s[4] += 4ull * w12_1_0;
+  s[5] += 4ull * w12_1_0;
+  s[2] += 2ull * w12_1_1;
+  s[11] += 16ull * w12_1_1;
+  s[1] += 2ull * w12_1_2;
+  s[10] += 16ull * w12_1_2;
+  s[7] += 4ull * w12_1_3;
+  const unsigned long long v33 = v(Idx<33>{});
+  const unsigned long long v34 = v(Idx<34>{});
+  const unsigned long long w13_0_0 = v33 + v34;
+  const unsigned long long w13_0_1 = v33 - v34;
+  s[0] += w13_0_0;
+  s[4] += 9ull * w13_0_0;
+  s[1] += 3ull * w13_0_1;
+  s[10] += 27ull * w13_0_1;
+}
+
+// s_k = sum_i p(i, y_i) phi_k(xi_i) in 64-bit integers.
+template <class V>
+__device__ __forceinline__ void jvec_fx(const int (&d)[13], const V& p, unsigned long long (&s)[13]) {
+  const int c0_0 = d[0];
+  const unsigned long long p0 = p(Idx<0>{}, c0_0);
+  s[0] = p0;
+  const int c1_0 = d[0] + d[6];
+  const int c1_z = d[3] + d[12];
+  const int y1_0_0 = c1_0 + c1_z;
+  const int y1_0_1 = c1_0 - c1_z;
+  const unsigned long long p5 = p(Idx<5>{}, y1_0_0);
+  const unsigned long long p6 = p(Idx<6>{}, y1_0_1);
+  const unsigned long long w1_0_0 = p5 + p6;
+  const unsigned long long w1_0_1 = p5 - p6;
+  s[0] += w1_0_0;
+  s[6] = w1_0_0;
+  s[3] = w1_0_1;
+  s[12] = w1_0_1;
+  const int c2_0 = d[0] + 4 * d[6];
+  const int c2_z = 2 * d[3] + 8 * d[12];
+  const int y2_0_0 = c2_0 + c2_z;
+  const int y2_0_1 = c2_0 - c2_z;
+  const unsigned long long p19 = p(Idx<19>{}, y2_0_0);
+  const unsigned long long p20 = p(Idx<20>{}, y2_0_1);
+  const unsigned long long w2_0_0 = p19 + p20;
+  const unsigned long long w2_0_1 = p19 - p20;
+  s[0] += w2_0_0;
+  s[6] += 4ull * w2_0_0;
+  s[3] += 2ull * w2_0_1;
+  s[12] += 8ull * w2_0_1;
+  const int c3_0 = d[0] + 9 * d[6];
+  const int c3_z = 3 * d[3] + 27 * d[12];
+  const int y3_0_0 = c3_0 + c3_z;
+  const int y3_0_1 = c3_0 - c3_z;
+  const unsigned long long p37 = p(Idx<37>{}, y3_0_0);
+  const unsigned long long p38 = p(Idx<38>{}, y3_0_1);
+  const unsigned long long w3_0_0 = p37 + p38;
+  const unsigned long long w3_0_1 = p37 - p38;
+  s[0] += w3_0_0;
+  s[6] += 9ull * w3_0_0;
+  s[3] += 3ull * w3_0_1;
+  s[12] += 27ull * w3_0_1;
+  const int c4_0 = d[0] + d[5];
+  const int c4_y = d[2] + d[11];
+  const int y4_0_0 = c4_0 + c4_y;
+  const int y4_0_1 = c4_0 - c4_y;
+  const unsigned long long p3 = p(Idx<3>{}, y4_0_0);
+  const unsigned long long p4 = p(Idx<4>{}, y4_0_1);
+  const unsigned long long w4_0_0 = p3 + p4;
+  const unsigned long long w4_0_1 = p3 - p4;
+  s[0] += w4_0_0;
+  s[5] = w4_0_0;
+  s[2] = w4_0_1;
+  s[11] = w4_0_1;
+  const int c5_0 = d[0] + 4 * d[5];
+  const int c5_y = 2 * d[2] + 8 * d[11];
+  const int y5_0_0 = c5_0 + c5_y;
+  const int y5_0_1 = c5_0 - c5_y;
+  const unsigned long long p17 = p(Idx<17>{}, y5_0_0);
+  const unsigned long long p18 = p(Idx<18>{}, y5_0_1);
+  const unsigned long long w5_0_0 = p17 + p18;
+  const unsigned long long w5_0_1 = p17 - p18;
+  s[0] += w5_0_0;
+  s[5] += 4ull * w5_0_0;
+  s[2] += 2ull * w5_0_1;
+  s[11] += 8ull * w5_0_1;
+  const int c6_0 = d[0] + 4 * d[5] + 4 * d[6];
+  const int c6_y = 2 * d[2] + 16 * d[11];
+  const int c6_z = 2 * d[3] + 16 * d[12];
+  const int c6_yz = 4 * d[9];
+  const int y6_0_0 = c6_0 + c6_y;
+  const int y6_0_1 = c6_0 - c6_y;
+  const int y6_0_2 = c6_z + c6_yz;
+  const int y6_0_3 = c6_z - c6_yz;
+  const int y6_1_0 = y6_0_1 + y6_0_3;
+  const int y6_1_1 = y6_0_1 - y6_0_3;
+  const int y6_1_2 = y6_0_0 + y6_0_2;
+  const int y6_1_3 = y6_0_0 - y6_0_2;
+  const unsigned long long p29 = p(Idx<29>{}, y6_1_2);
+  const unsigned long long p30 = p(Idx<30>{}, y6_1_1);
+  const unsigned long long p31 = p(Idx<31>{}, y6_1_3);
+  const unsigned long long p32 = p(Idx<32>{}, y6_1_0);
+  const unsigned long long w6_0_0 = p31 + p30;
+  const unsigned long long w6_0_1 = p31 - p30;
+  const unsigned long long w6_0_2 = p29 + p32;
+  const unsigned long long w6_0_3 = p29 - p32;
+  const unsigned long long w6_1_0 = w6_0_2 + w6_0_0;
+  const unsigned long long w6_1_1 = w6_0_2 - w6_0_0;
+  const unsigned long long w6_1_2 = w6_0_3 + w6_0_1;
+  const unsigned long long w6_1_3 = w6_0_3 - w6_0_1;
+  s[0] += w6_1_0;
+  s[5] += 4ull * w6_1_0;
+  s[6] += 4ull * w6_1_0;
+  s[3] += 2ull * w6_1_1;
+  s[12] += 16ull * w6_1_1;
+  s[2] += 2ull * w6_1_2;
+  s[11] += 16ull * w6_1_2;
+  s[9] = 4ull * w6_1_3;
+  const int c7_0 = d[0] + 9 * d[5];
+  const int c7_y = 3 * d[2] + 27 * d[11];
+  const int y7_0_0 = c7_0 + c7_y;
+  const int y7_0_1 = c7_0 - c7_y;
+  const unsigned long long p35 = p(Idx<35>{}, y7_0_0);
+  const unsigned long long p36 = p(Idx<36>{}, y7_0_1);
+  const unsigned long long w7_0_0 = p35 + p36;
+  const unsigned long long w7_0_1 = p35 - p36;
+  s[0] += w7_0_0;
+  s[5] += 9ull * w7_0_0;
+  s[2] += 3ull * w7_0_1;
+  s[11] += 27ull * w7_0_1;
+  const int c8_0 = d[0] + d[4];
+  const int c8_x = d[1] + d[10];
+  const int y8_0_0 = c8_0 + c8_x;
+  const int y8_0_1 = c8_0 - c8_x;
+  const unsigned long long p1 = p(Idx<1>{}, y8_0_0);
+  const unsigned long long p2 = p(Idx<2>{}, y8_0_1);
+  const unsigned long long w8_0_0 = p1 + p2;
+  const unsigned long long w8_0_1 = p1 - p2;
+  s[0] += w8_0_0;
+  s[4] = w8_0_0;
+  s[1] = w8_0_1;
+  s[10] = w8_0_1;
+  const int c9_0 = d[0] + d[4] + d[5] + d[6];
+  const int c9_x = d[1] + 3 * d[10];
+  const int c9_y = d[2] + 3 * d[11];
+  const int c9_z = d[3] + 3 * d[12];
+  const int c9_xy = d[7];
+  const int c9_xz = d[8];
+  const int c9_yz = d[9];
+  const int y9_0_0 = c9_0 + c9_x;
+  const int y9_0_1 = c9_0 - c9_x;
+  const int y9_0_2 = c9_y + c9_xy;
+  const int y9_0_3 = c9_y - c9_xy;
+  const int y9_0_6 = c9_z + c9_xz;
+  const int y9_0_7 = c9_z - c9_xz;
+  const int y9_1_0 = y9_0_1 + y9_0_3;
+  const int y9_1_1 = y9_0_1 - y9_0_3;
+  const int y9_1_2 = y9_0_7 + c9_yz;
+  const int y9_1_3 = y9_0_7 - c9_yz;
+  const int y9_1_4 = y9_0_0 + y9_0_2;
+  const int y9_1_5 = y9_0_0 - y9_0_2;
+  const int y9_1_6 = y9_0_6 + c9_yz;
+  const int y9_1_7 = y9_0_6 - c9_yz;
+  const int y9_2_0 = y9_1_1 + y9_1_3;
+  const int y9_2_1 = y9_1_1 - y9_1_3;
+  const int y9_2_2 = y9_1_0 + y9_1_2;
+  const int y9_2_3 = y9_1_0 - y9_1_2;
+  const int y9_2_4 = y9_1_5 + y9_1_7;
+  const int y9_2_5 = y9_1_5 - y9_1_7;
+  const int y9_2_6 = y9_1_4 + y9_1_6;
+  const int y9_2_7 = y9_1_4 - y9_1_6;
+  const unsigned long long p7 = p(Idx<7>{}, y9_2_6);
+  const unsigned long long p8 = p(Idx<8>{}, y9_2_1);
+  const unsigned long long p9 = p(Idx<9>{}, y9_2_7);
+  const unsigned long long p10 = p(Idx<10>{}, y9_2_0);
+  const unsigned long long p11 = p(Idx<11>{}, y9_2_4);
+  const unsigned long long p12 = p(Idx<12>{}, y9_2_3);
+  const unsigned long long p13 = p(Idx<13>{}, y9_2_2);
+  const unsigned long long p14 = p(Idx<14>{}, y9_2_5);
+  const unsigned long long w9_0_0 = p14 + p8;
+  const unsigned long long w9_0_1 = p14 - p8;
+  const unsigned long long w9_0_2 = p11 + p10;
+  const unsigned long long w9_0_3 = p11 - p10;
+  const unsigned long long w9_0_4 = p9 + p12;
+  const unsigned long long w9_0_5 = p9 - p12;
+  const unsigned long long w9_0_6 = p7 + p13;
+  const unsigned long long w9_0_7 = p7 - p13;
+  const unsigned long long w9_1_0 = w9_0_4 + w9_0_0;
+  const unsigned long long w9_1_1 = w9_0_4 - w9_0_0;
+  const unsigned long long w9_1_2 = w9_0_6 + w9_0_2;
+  const unsigned long long w9_1_3 = w9_0_6 - w9_0_2;
+  const unsigned long long w9_1_4 = w9_0_5 + w9_0_1;
+  const unsigned long long w9_1_5 = w9_0_5 - w9_0_1;
+  const unsigned long long w9_1_6 = w9_0_7 + w9_0_3;
+  const unsigned long long w9_1_7 = w9_0_7 - w9_0_3;
+  const unsigned long long w9_2_0 = w9_1_2 + w9_1_0;
+  const unsigned long long w9_2_1 = w9_1_2 - w9_1_0;
+  const unsigned long long w9_2_2 = w9_1_3 + w9_1_1;
+  const unsigned long long w9_2_3 = w9_1_3 - w9_1_1;
+  const unsigned long long w9_2_4 = w9_1_6 + w9_1_4;
+  const unsigned long long w9_2_5 = w9_1_6 - w9_1_4;
+  const unsigned long long w9_2_6 = w9_1_7 + w9_1_5;
+  const unsigned long long w9_2_7 = w9_1_7 - w9_1_5;
+  s[0] += w9_2_0;
+  s[4] += w9_2_0;
+  s[5] += w9_2_0;
+  s[6] += w9_2_0;
+  s[3] += w9_2_1;
+  s[12] += 3ull * w9_2_1;
+  s[2] += w9_2_2;
+  s[11] += 3ull * w9_2_2;
+  s[9] += w9_2_3;
+  s[1] += w9_2_4;
+  s[10] += 3ull * w9_2_4;
+  s[8] = w9_2_5;
+  s[7] = w9_2_6;
+  const int c10_0 = d[0] + 4 * d[4];
+  const int c10_x = 2 * d[1] + 8 * d[10];
+  const int y10_0_0 = c10_0 + c10_x;
+  const int y10_0_1 = c10_0 - c10_x;
+  const unsigned long long p15 = p(Idx<15>{}, y10_0_0);
+  const unsigned long long p16 = p(Idx<16>{}, y10_0_1);
+  const unsigned long long w10_0_0 = p15 + p16;
+  const unsigned long long w10_0_1 = p15 - p16;
+  s[0] += w10_0_0;
+  s[4] += 4ull * w10_0_0;
+  s[1] += 2ull * w10_0_1;
+  s[10] += 8ull * w10_0_1;
+  const int c11_0 = d[0] + 4 * d[4] + 4 * d[6];
+  const int c11_x = 2 * d[1] + 16 * d[10];
+  const int c11_z = 2 * d[3] + 16 * d[12];
+  const int c11_xz = 4 * d[8];
+  const int y11_0_0 = c11_0 + c11_x;
+  const int y11_0_1 = c11_0 - c11_x;
+  const int y11_0_2 = c11_z + c11_xz;
+  const int y11_0_3 = c11_z - c11_xz;
+  const int y11_1_0 = y11_0_1 + y11_0_3;
+  const int y11_1_1 = y11_0_1 - y11_0_3;
+  const int y11_1_2 = y11_0_0 + y11_0_2;
+  const int y11_1_3 = y11_0_0 - y11_0_2;
+  const unsigned long long p25 = p(Idx<25>{}, y11_1_2);
+  const unsigned long long p26 = p(Idx<26>{}, y11_1_1);
+  const unsigned long long p27 = p(Idx<27>{}, y11_1_3);
+  const unsigned long long p28 = p(Idx<28>{}, y11_1_0);
+  const unsigned long long w11_0_0 = p27 + p26;
+  const unsigned long long w11_0_1 = p27 - p26;
+  const unsigned long long w11_0_2 = p25 + p28;
+  const unsigned long long w11_0_3 = p25 - p28;
+  const unsigned long long w11_1_0 = w11_0_2 + w11_0_0;
+  const unsigned long long w11_1_1 = w11_0_2 - w11_0_0;
+  const unsigned long long w11_1_2 = w11_0_3 + w11_0_1;
+  const unsigned long long w11_1_3 = w11_0_3 - w11_0_1;
+  s[0] += w11_1_0;
+  s[4] += 4ull * w11_1_0;
+  s[6] += 4ull * w11_1_0;
+  s[3] += 2ull * w11_1_1;
+  s[12] += 16ull * w11_1_1;
+  s[1] += 2ull * w11_1_2;
+  s[10] += 16ull * w11_1_2;
+  s[8] += 4ull * w11_1_3;
+  const int c12_0 = d[0] + 4 * d[4] + 4 * d[5];
+  const int c12_x = 2 * d[1] + 16 * d[10];
+  const int c12_y = 2 * d[2] + 16 * d[11];
+  const int c12_xy = 4 * d[7];
+  const int y12_0_0 = c12_0 + c12_x;
+  const int y12_0_1 = c12_0 - c12_x;
+  const int y12_0_2 = c12_y + c12_xy;
+  const int y12_0_3 = c12_y - c12_xy;
+  const int y12_1_0 = y12_0_1 + y12_0_3;
+  const int y12_1_1 = y12_0_1 - y12_0_3;
+  const int y12_1_2 = y12_0_0 + y12_0_2;
+  const int y12_1_3 = y12_0_0 - y12_0_2;
+  const unsigned long long p21 = p(Idx<21>{}, y12_1_2);
+  const unsigned long long p22 = p(Idx<22>{}, y12_1_1);
+  const unsigned long long p23 = p(Idx<23>{}, y12_1_3);
+  const unsigned long long p24 = p(Idx<24>{}, y12_1_0);
+  const unsigned long long w12_0_0 = p23 + p22;
+  const unsigned long long w12_0_1 = p23 - p22;
+  const unsigned long long w12_0_2 = p21 + p24;
+  const unsigned long long w12_0_3 = p21 - p24;
+  const unsigned long long w12_1_0 = w12_0_2 + w12_0_0;
+  const unsigned long long w12_1_1 = w12_0_2 - w12_0_0;
+  const unsigned long long w12_1_2 = w12_0_3 + w12_0_1;
+  const unsigned long long w12_1_3 = w12_0_3 - w12_0_1;
+  s[0] += w12_1_0;
+  s[4] += 4ull * w12_1_0;
+  s[5] += 4ull * w12_1_0;
+  s[2] += 2ull * w12_1_1;
+  s[11] += 16ull * w12_1_1;
+  s[1] += 2ull * w12_1_2;
+  s[10] += 16ull * w12_1_2;
+  s[7] += 4ull * w12_1_3;
+  const int c13_0 = d[0] + 9 * d[4];
+  const int c13_x = 3 * d[1] + 27 * d[10];
+  const int y13_0_0 = c13_0 + c13_x;
+  const int y13_0_1 = c13_0 - c13_x;
+  const unsigned long long p33 = p(Idx<33>{}, y13_0_0);
+  const unsigned long long p34 = p(Idx<34>{}, y13_0_1);
+  const unsigned long long w13_0_0 = p33 + p34;
+  const unsigned long long w13_0_1 = p33 - p34;
+  s[0] += w13_0_0;
+  s[4] += 9ull * w13_0_0;
+  s[1] += 3ull * w13_0_1;
+  s[10] += 27ull * w13_0_1;
+}
+
+// s_k = sum_i v(i) phi_k(xi_i) in 64-bit integers (the nine z-even k, values mirror-symmetric in z).
+template <class V>
+__device__ __forceinline__ void sums_fx2d(const V& v, unsigned long long (&s)[9]) {
+  const unsigned long long v0 = v(Idx<0>{});
+  s[0] = v0;
+  const unsigned long long v5 = v(Idx<5>{});
+  s[0] += 2ull * v5;
+  s[5] = 2ull * v5;
+  const unsigned long long v19 = v(Idx<19>{});
+  s[0] += 2ull * v19;
+  s[5] += 8ull * v19;
+  const unsigned long long v37 = v(Idx<37>{});
+  s[0] += 2ull * v37;
+  s[5] += 18ull * v37;
+  const unsigned long long v3 = v(Idx<3>{});
+  const unsigned long long v4 = v(Idx<4>{});
+  const unsigned long long w4_0_0 = v3 + v4;
+  const unsigned long long w4_0_1 = v3 - v4;
+  s[0] += w4_0_0;
+  s[4] = w4_0_0;
+  s[2] = w4_0_1;
+  s[8] = w4_0_1;
+  const unsigned long long v17 = v(Idx<17>{});
+  const unsigned long long v18 = v(Idx<18>{});
+  const unsigned long long w5_0_0 = v17 + v18;
+  const unsigned long long w5_0_1 = v17 - v18;
+  s[0] += w5_0_0;
+  s[4] += 4ull * w5_0_0;
+  s[2] += 2ull * w5_0_1;
+  s[8] += 8ull * w5_0_1;
+  const unsigned long long v29 = v(Idx<29>{});
+  const unsigned long long v32 = v(Idx<32>{});
+  const unsigned long long w6_0_0 = v29 + v32;
+  const unsigned long long w6_0_1 = v29 - v32;
+  s[0] += 2ull * w6_0_0;
+  s[4] += 8ull * w6_0_0;
+  s[5] += 8ull * w6_0_0;
+  s[2] += 4ull * w6_0_1;
+  s[8] += 32ull * w6_0_1;
+  const unsigned long long v35 = v(Idx<35>{});
+  const unsigned long long v36 = v(Idx<36>{});
+  const unsigned long long w7_0_0 = v35 + v36;
+  const unsigned long long w7_0_1 = v35 - v36;
+  s[0] += w7_0_0;
+  s[4] += 9ull * w7_0_0;
+  s[2] += 3ull * w7_0_1;
+  s[8] += 27ull * w7_0_1;
+  const unsigned long long v1 = v(Idx<1>{});
+  const unsigned long long v2 = v(Idx<2>{});
+  const unsigned long long w8_0_0 = v1 + v2;
+  const unsigned long long w8_0_1 = v1 - v2;
+  s[0] += w8_0_0;
+  s[3] = w8_0_0;
+  s[1] = w8_0_1;
+  s[7] = w8_0_1;
+  const unsigned long long v7 = v(Idx<7>{});
+  const unsigned long long v10 = v(Idx<10>{});
+  const unsigned long long v11 = v(Idx<11>{});
+  const unsigned long long v13 = v(Idx<13>{});
+  const unsigned long long w9_0_0 = v11 + v10;
+  const unsigned long long w9_0_1 = v11 - v10;
+  const unsigned long long w9_0_2 = v7 + v13;
+  const unsigned long long w9_0_3 = v7 - v13;
+  const unsigned long long w9_1_0 = w9_0_2 + w9_0_0;
+  const unsigned long long w9_1_1 = w9_0_2 - w9_0_0;
+  const unsigned long long w9_1_2 = w9_0_3 + w9_0_1;
+  const unsigned long long w9_1_3 = w9_0_3 - w9_0_1;
+  s[0] += 2ull * w9_1_0;
+  s[3] += 2ull * w9_1_0;
+  s[4] += 2ull * w9_1_0;
+  s[5] += 2ull * w9_1_0;
+  s[2] += 2ull * w9_1_1;
+  s[8] += 6ull * w9_1_1;
+  s[1] += 2ull * w9_1_2;
+  s[7] += 6ull * w9_1_2;
+  s[6] = 2ull * w9_1_3;
+  const unsigned long long v15 = v(Idx<15>{});
+  const unsigned long long v16 = v(Idx<16>{});
+  const unsigned long long w10_0_0 = v15 + v16;
+  const unsigned long long w10_0_1 = v15 - v16;
+  s[0] += w10_0_0;
+  s[3] += 4ull * w10_0_0;
+  s[1] += 2ull * w10_0_1;
+  s[7] += 8ull * w10_0_1;
+  const unsigned long long v25 = v(Idx<25>{});
+  const unsigned long long v28 = v(Idx<28>{});
+  const unsigned long long w11_0_0 = v25 + v28;
+  const unsigned long long w11_0_1 = v25 - v28;
+  s[0] += 2ull * w11_0_0;
+  s[3] += 8ull * w11_0_0;
+  s[5] += 8ull * w11_0_0;
+  s[1] += 4ull * w11_0_1;
+  s[7] += 32ull * w11_0_1;
+  const unsigned long long v21 = v(Idx<21>{});
+  const unsigned long long v22 = v(Idx<22>{});
+  const unsigned long long v23 = v(Idx<23>{});
+  const unsigned long long v24 = v(Idx<24>{});
+  const unsigned long long w12_0_0 = v23 + v22;
+  const unsigned long long w12_0_1 = v23 - v22;
+  const unsigned long long w12_0_2 = v21 + v24;
+  const unsigned long long w12_0_3 = v21 - v24;
+  const unsigned long long w12_1_0 = w12_0_2 + w12_0_0;
+  const unsigned long long w12_1_1 = w12_0_2 - w12_0_0;
+  const unsigned long long w12_1_2 = w12_0_3 + w12_0_1;
+  const unsigned long long w12_1_3 = w12_0_3 - w12_0_1;
+  s[0] += w12_1_0;
+  s[3] += 4ull * w12_1_0;
+  s[4] += 4ull * w12_1_0;
+  s[2] += 2ull * w12_1_1;
+  s[8] += 16ull * w12_1_1;
+  s[1] += 2ull * w12_1_2;
+  s[7] += 16ull * w12_1_2;
+  s[6] += 4ull * w12_1_3;
+  const unsigned long long v33 = v(Idx<33>{});
+  const unsigned long long v34 = v(Idx<34>{});
+  const unsigned long long w13_0_0 = v33 + v34;
+  const unsigned long long w13_0_1 = v33 - v34;
+  s[0] += w13_0_0;
+  s[3] += 9ull * w13_0_0;
+  s[1] += 3ull * w13_0_1;
+  s[7] += 27ull * w13_0_1;
+}
+
+// s_k = sum_i p(i, y_i) phi_k(xi_i) in 64-bit integers (the nine z-even k, values mirror-symmetric in z).
+template <class V>
+__device__ __forceinline__ void jvec_fx2d(const int (&d)[9], const V& p, unsigned long long (&s)[9]) {
+  const int c0_0 = d[0];
+  const unsigned long long p0 = p(Idx<0>{}, c0_0);
+  s[0] = p0;
+  const int c1_0 = d[0] + d[5];
+  const unsigned long long p5 = p(Idx<5>{}, c1_0);
+  s[0] += 2ull * p5;
+  s[5] = 2ull * p5;
+  const int c2_0 = d[0] + 4 * d[5];
+  const unsigned long long p19 = p(Idx<19>{}, c2_0);
+  s[0] += 2ull * p19;
+  s[5] += 8ull * p19;
+  const int c3_0 = d[0] + 9 * d[5];
+  const unsigned long long p37 = p(Idx<37>{}, c3_0);
+  s[0] += 2ull * p37;
+  s[5] += 18ull * p37;
+  const int c4_0 = d[0] + d[4];
+  const int c4_y = d[2] + d[8];
+  const int y4_0_0 = c4_0 + c4_y;
+  const int y4_0_1 = c4_0 - c4_y;
+  const unsigned long long p3 = p(Idx<3>{}, y4_0_0);
+  const unsigned long long p4 = p(Idx<4>{}, y4_0_1);
+  const unsigned long long w4_0_0 = p3 + p4;
+  const unsigned long long w4_0_1 = p3 - p4;
+  s[0] += w4_0_0;
+  s[4] = w4_0_0;
+  s[2] = w4_0_1;
+  s[8] = w4_0_1;
+  const int c5_0 = d[0] + 4 * d[4];
+  const int c5_y = 2 * d[2] + 8 * d[8];
+  const int y5_0_0 = c5_0 + c5_y;
+  const int y5_0_1 = c5_0 - c5_y;
+  const unsigned long long p17 = p(Idx<17>{}, y5_0_0);
+  const unsigned long long p18 = p(Idx<18>{}, y5_0_1);
+  const unsigned long long w5_0_0 = p17 + p18;
+  const unsigned long long w5_0_1 = p17 - p18;
+  s[0] += w5_0_0;
+  s[4] += 4ull * w5_0_0;
+  s[2] += 2ull * w5_0_1;
+  s[8] += 8ull * w5_0_1;
+  const int c6_0 = d[0] + 4 * d[4] + 4 * d[5];
+  const int c6_y = 2 * d[2] + 16 * d[8];
+  const int y6_0_0 = c6_0 + c6_y;
+  const int y6_0_1 = c6_0 - c6_y;
+  const unsigned long long p29 = p(Idx<29>{}, y6_0_0);
+  const unsigned long long p32 = p(Idx<32>{}, y6_0_1);
+  const unsigned long long w6_0_0 = p29 + p32;
+  const unsigned long long w6_0_1 = p29 - p32;
+  s[0] += 2ull * w6_0_0;
+  s[4] += 8ull * w6_0_0;
+  s[5] += 8ull * w6_0_0;
+  s[2] += 4ull * w6_0_1;
+  s[8] += 32ull * w6_0_1;
+  const int c7_0 = d[0] + 9 * d[4];
+  const int c7_y = 3 * d[2] + 27 * d[8];
+  const int y7_0_0 = c7_0 + c7_y;
+  const int y7_0_1 = c7_0 - c7_y;
+  const unsigned long long p35 = p(Idx<35>{}, y7_0_0);
+  const unsigned long long p36 = p(Idx<36>{}, y7_0_1);
+  const unsigned long long w7_0_0 = p35 + p36;
+  const unsigned long long w7_0_1 = p35 - p36;
+  s[0] += w7_0_0;
+  s[4] += 9ull * w7_0_0;
+  s[2] += 3ull * w7_0_1;
+  s[8] += 27ull * w7_0_1;
+  const int c8_0 = d[0] + d[3];
+  const int c8_x = d[1] + d[7];
+  const int y8_0_0 = c8_0 + c8_x;
+  const int y8_0_1 = c8_0 - c8_x;
+  const unsigned long long p1 = p(Idx<1>{}, y8_0_0);
+  const unsigned long long p2 = p(Idx<2>{}, y8_0_1);
+  const unsigned long long w8_0_0 = p1 + p2;
+  const unsigned long long w8_0_1 = p1 - p2;
+  s[0] += w8_0_0;
+  s[3] = w8_0_0;
+  s[1] = w8_0_1;
+  s[7] = w8_0_1;
+  const int c9_0 = d[0] + d[3] + d[4] + d[5];
+  const int c9_x = d[1] + 3 * d[7];
+  const int c9_y = d[2] + 3 * d[8];
+  const int c9_xy = d[6];
+  const int y9_0_0 = c9_0 + c9_x;
+  const int y9_0_1 = c9_0 - c9_x;
+  const int y9_0_2 = c9_y + c9_xy;
+  const int y9_0_3 = c9_y - c9_xy;
+  const int y9_1_0 = y9_0_1 + y9_0_3;
+  const int y9_1_1 = y9_0_1 - y9_0_3;
+  const int y9_1_2 = y9_0_0 + y9_0_2;
+  const int y9_1_3 = y9_0_0 - y9_0_2;
+  const unsigned long long p7 = p(Idx<7>{}, y9_1_2);
+  const unsigned long long p10 = p(Idx<10>{}, y9_1_1);
+  const unsigned long long p11 = p(Idx<11>{}, y9_1_3);
+  const unsigned long long p13 = p(Idx<13>{}, y9_1_0);
+  const unsigned long long w9_0_0 = p11 + p10;
+  const unsigned long long w9_0_1 = p11 - p10;
+  const unsigned long long w9_0_2 = p7 + p13;
+  const unsigned long long w9_0_3 = p7 - p13;
+  const unsigned long long w9_1_0 = w9_0_2 + w9_0_0;
+  const unsigned long long w9_1_1 = w9_0_2 - w9_0_0;
+  const unsigned long long w9_1_2 = w9_0_3 + w9_0_1;
+  const unsigned long long w9_1_3 = w9_0_3 - w9_0_1;
+  s[0] += 2ull * w9_1_0;
+  s[3] += 2ull * w9_1_0;
+  s[4] += 2ull * w9_1_0;
+  s[5] += 2ull * w9_1_0;
+  s[2] += 2ull * w9_1_1;
+  s[8] += 6ull * w9_1_1;
+  s[1] += 2ull * w9_1_2;
+  s[7] += 6ull * w9_1_2;
+  s[6] = 2ull * w9_1_3;
+  const int c10_0 = d[0] + 4 * d[3];
+  const int c10_x = 2 * d[1] + 8 * d[7];
+  const int y10_0_0 = c10_0 + c10_x;
+  const int y10_0_1 = c10_0 - c10_x;
+  const unsigned long long p15 = p(Idx<15>{}, y10_0_0);
+  const unsigned long long p16 = p(Idx<16>{}, y10_0_1);
+  const unsigned long long w10_0_0 = p15 + p16;
+  const unsigned long long w10_0_1 = p15 - p16;
+  s[0] += w10_0_0;
+  s[3] += 4ull * w10_0_0;
+  s[1] += 2ull * w10_0_1;
+  s[7] += 8ull * w10_0_1;
+  const int c11_0 = d[0] + 4 * d[3] + 4 * d[5];
+  const int c11_x = 2 * d[1] + 16 * d[7];
+  const int y11_0_0 = c11_0 + c11_x;
+  const int y11_0_1 = c11_0 - c11_x;
+  const unsigned long long p25 = p(Idx<25>{}, y11_0_0);
+  const unsigned long long p28 = p(Idx<28>{}, y11_0_1);
+  const unsigned long long w11_0_0 = p25 + p28;
+  const unsigned long long w11_0_1 = p25 - p28;
+  s[0] += 2ull * w11_0_0;
+  s[3] += 8ull * w11_0_0;
+  s[5] += 8ull * w11_0_0;
+  s[1] += 4ull * w11_0_1;
+  s[7] += 32ull * w11_0_1;
+  const int c12_0 = d[0] + 4 * d[3] + 4 * d[4];
+  const int c12_x = 2 * d[1] + 16 * d[7];
+  const int c12_y = 2 * d[2] + 16 * d[8];
+  const int c12_xy = 4 * d[6];
+  const int y12_0_0 = c12_0 + c12_x;
+  const int y12_0_1 = c12_0 - c12_x;
+  const int y12_0_2 = c12_y + c12_xy;
+  const int y12_0_3 = c12_y - c12_xy;
+  const int y12_1_0 = y12_0_1 + y12_0_3;
+  const int y12_1_1 = y12_0_1 - y12_0_3;
+  const int y12_1_2 = y12_0_0 + y12_0_2;
+  const int y12_1_3 = y12_0_0 - y12_0_2;
+  const unsigned long long p21 = p(Idx<21>{}, y12_1_2);
+  const unsigned long long p22 = p(Idx<22>{}, y12_1_1);
+  const unsigned long long p23 = p(Idx<23>{}, y12_1_3);
+  const unsigned long long p24 = p(Idx<24>{}, y12_1_0);
+  const unsigned long long w12_0_0 = p23 + p22;
+  const unsigned long long w12_0_1 = p23 - p22;
+  const unsigned long long w12_0_2 = p21 + p24;
+  const unsigned long long w12_0_3 = p21 - p24;
+  const unsigned long long w12_1_0 = w12_0_2 + w12_0_0;
+  const unsigned long long w12_1_1 = w12_0_2 - w12_0_0;
+  const unsigned long long w12_1_2 = w12_0_3 + w12_0_1;
+  const unsigned long long w12_1_3 = w12_0_3 - w12_0_1;
+  s[0] += w12_1_0;
+  s[3] += 4ull * w12_1_0;
+  s[4] += 4ull * w12_1_0;
+  s[2] += 2ull * w12_1_1;
+  s[8] += 16ull * w12_1_1;
+  s[1] += 2ull * w12_1_2;
+  s[7] += 16ull * w12_1_2;
+  s[6] += 4ull * w12_1_3;
+  const int c13_0 = d[0] + 9 * d[3];
+  const int c13_x = 3 * d[1] + 27 * d[7];
+  const int y13_0_0 = c13_0 + c13_x;
+  const int y13_0_1 = c13_0 - c13_x;
+  const unsigned long long p33 = p(Idx<33>{}, y13_0_0);
+  const unsigned long long p34 = p(Idx<34>{}, y13_0_1);
+  const unsigned long long w13_0_0 = p33 + p34;
+  const unsigned long long w13_0_1 = p33 - p34;
+  s[0] += w13_0_0;
+  s[3] += 9ull * w13_0_0;
+  s[1] += 3ull * w13_0_1;
+  s[7] += 27ull * w13_0_1;
+}
+
+// 2^(j/1024) in units of 2^-55, j = 0..1023, each the integer nearest the exact value.
+__device__ const unsigned long long kExp2Fixed[1024] = {
+    36028797018963968ull, 36053193223259766ull, 36077605946974287ull, 36102035201293337ull,
+    36126480997410295ull, 36150943346526120ull, 36175422259849356ull, 36199917748596135ull,
+    36224429823990187ull, 36248958497262839ull, 36273503779653025ull, 36298065682407286ull,
+    36322644216779783ull, 36347239394032294ull, 36371851225434223ull, 36396479722262608ull,
+    36421124895802119ull, 36445786757345070ull, 36470465318191420ull, 36495160589648779ull,
+    36519872583032416ull, 36544601309665260ull, 36569346780877907ull, 36594109008008627ull,
+    36618888002403366ull, 36643683775415753ull, 36668496338407104ull, 36693325702746431ull,
+    36718171879810441ull, 36743034880983547ull, 36767914717657869ull, 36792811401233241ull,
+    36817724943117218ull, 36842655354725077ull, 36867602647479827ull, 36892566832812210ull,
+    36917547922160709ull, 36942545926971552ull, 36967560858698718ull, 36992592728803942ull,
+    37017641548756718ull, 37042707330034310ull, 37067790084121750ull, 37092889822511850ull,
+    37118006556705201ull, 37143140298210185ull, 37168291058542973ull, 37193458849227536ull,
+    37218643681795648ull, 37243845567786892ull, 37269064518748664ull, 37294300546236179ull,
+    37319553661812477ull, 37344823877048427ull, 37370111203522734ull, 37395415652821942ull,
+    37420737236540442ull, 37446075966280475ull, 37471431853652138ull, 37496804910273390ull,
+    37522195147770057ull, 37547602577775838ull, 37573027211932307ull, 37598469061888924ull,
+    37623928139303035ull, 37649404455839880ull, 37674898023172599ull, 37700408852982234ull,
+    37725936956957739ull, 37751482346795981ull, 37777045034201749ull, 37802625030887757ull,
+    37828222348574650ull, 37853836998991009ull, 37879468993873356ull, 37905118344966163ull,
+    37930785064021853ull, 37956469162800805ull, 37982170653071364ull, 38007889546609843ull,
+    38033625855200528ull, 38059379590635686ull, 38085150764715569ull, 38110939389248418ull,
+    38136745476050469ull, 38162569036945963ull, 38188410083767143ull, 38214268628354266ull,
+    38240144682555608ull, 38266038258227464ull, 38291949367234161ull, 38317878021448059ull,
+    38343824232749554ull, 38369788013027090ull, 38395769374177160ull, 38421768328104313ull,
+    38447784886721157ull, 38473819061948369ull, 38499870865714696ull, 38525940309956962ull,
+    38552027406620076ull, 38578132167657034ull, 38604254605028925ull, 38630394730704939ull,
+    38656552556662368ull, 38682728094886617ull, 38708921357371205ull, 38735132356117773ull,
+    38761361103136088ull, 38787607610444049ull, 38813871890067695ull, 38840153954041206ull,
+    38866453814406910ull, 38892771483215290ull, 38919106972524991ull, 38945460294402821ull,
+    38971831460923758ull, 38998220484170959ull, 39024627376235760ull, 39051052149217687ull,
+    39077494815224457ull, 39103955386371987ull, 39130433874784397ull, 39156930292594017ull,
+    39183444651941392ull, 39209976964975288ull, 39236527243852698ull, 39263095500738845ull,
+    39289681747807191ull, 39316285997239440ull, 39342908261225546ull, 39369548551963716ull,
+    39396206881660417ull, 39422883262530381ull, 39449577706796612ull, 39476290226690390ull,
+    39503020834451278ull, 39529769542327125ull, 39556536362574074ull, 39583321307456568ull,
+    39610124389247355ull, 39636945620227490ull, 39663785012686348ull, 39690642578921624ull,
+    39717518331239338ull, 39744412281953846ull, 39771324443387840ull, 39798254827872358ull,
+    39825203447746787ull, 39852170315358868ull, 39879155443064706ull, 39906158843228769ull,
+    39933180528223901ull, 39960220510431321ull, 39987278802240634ull, 40014355416049833ull,
+    40041450364265306ull, 40068563659301843ull, 40095695313582640ull, 40122845339539303ull,
+    40150013749611860ull, 40177200556248758ull, 40204405771906877ull, 40231629409051529ull,
+    40258871480156469ull, 40286131997703897ull, 40313410974184465ull, 40340708422097283ull,
+    40368024353949926ull, 40395358782258435ull, 40422711719547330ull, 40450083178349609ull,
+    40477473171206757ull, 40504881710668751ull, 40532308809294067ull, 40559754479649683ull,
+    40587218734311090ull, 40614701585862290ull, 40642203046895808ull, 40669723130012696ull,
+    40697261847822538ull, 40724819212943457ull, 40752395238002120ull, 40779989935633742ull,
+    40807603318482097ull, 40835235399199518ull, 40862886190446906ull, 40890555704893735ull,
+    40918243955218058ull, 40945950954106513ull, 40973676714254328ull, 41001421248365328ull,
+    41029184569151939ull, 41056966689335197ull, 41084767621644748ull, 41112587378818863ull,
+    41140425973604434ull, 41168283418756986ull, 41196159727040681ull, 41224054911228324ull,
+    41251968984101370ull, 41279901958449926ull, 41307853847072763ull, 41335824662777315ull,
+    41363814418379690ull, 41391823126704676ull, 41419850800585742ull, 41447897452865047ull,
+    41475963096393449ull, 41504047744030505ull, 41532151408644479ull, 41560274103112352ull,
+    41588415840319820ull, 41616576633161307ull, 41644756494539969ull, 41672955437367697ull,
+    41701173474565125ull, 41729410619061637ull, 41757666883795373ull, 41785942281713232ull,
+    41814236825770879ull, 41842550528932754ull, 41870883404172074ull, 41899235464470842ull,
+    41927606722819849ull, 41955997192218686ull, 41984406885675743ull, 42012835816208221ull,
+    42041283996842133ull, 42069751440612314ull, 42098238160562425ull, 42126744169744959ull,
+    42155269481221248ull, 42183814108061466ull, 42212378063344640ull, 42240961360158652ull,
+    42269564011600245ull, 42298186030775033ull, 42326827430797501ull, 42355488224791017ull,
+    42384168425887834ull, 42412868047229097ull, 42441587101964849ull, 42470325603254038ull,
+    42499083564264524ull, 42527860998173079ull, 42556657918165402ull, 42585474337436117ull,
+    42614310269188785ull, 42643165726635905ull, 42672040722998926ull, 42700935271508246ull,
+    42729849385403224ull, 42758783077932183ull, 42787736362352417ull, 42816709251930197ull,
+    42845701759940777ull, 42874713899668401ull, 42903745684406305ull, 42932797127456730ull,
+    42961868242130922ull, 42990959041749141ull, 43020069539640668ull, 43049199749143808ull,
+    43078349683605898ull, 43107519356383313ull, 43136708780841472ull, 43165917970354845ull,
+    43195146938306956ull, 43224395698090395ull, 43253664263106818ull, 43282952646766955ull,
+    43312260862490618ull, 43341588923706708ull, 43370936843853214ull, 43400304636377230ull,
+    43429692314734951ull, 43459099892391686ull, 43488527382821861ull, 43517974799509026ull,
+    43547442155945862ull, 43576929465634185ull, 43606436742084954ull, 43635963998818276ull,
+    43665511249363414ull, 43695078507258792ull, 43724665786052001ull, 43754273099299806ull,
+    43783900460568149ull, 43813547883432162ull, 43843215381476167ull, 43872902968293683ull,
+    43902610657487437ull, 43932338462669364ull, 43962086397460617ull, 43991854475491572ull,
+    44021642710401836ull, 44051451115840250ull, 44081279705464898ull, 44111128492943111ull,
+    44140997491951477ull, 44170886716175842ull, 44200796179311322ull, 44230725895062304ull,
+    44260675877142455ull, 44290646139274730ull, 44320636695191374ull, 44350647558633931ull,
+    44380678743353251ull, 44410730263109493ull, 44440802131672135ull, 44470894362819979ull,
+    44501006970341156ull, 44531139968033134ull, 44561293369702723ull, 44591467189166083ull,
+    44621661440248729ull, 44651876136785537ull, 44682111292620752ull, 44712366921607992ull,
+    44742643037610258ull, 44772939654499935ull, 44803256786158805ull, 44833594446478047ull,
+    44863952649358246ull, 44894331408709402ull, 44924730738450933ull, 44955150652511679ull,
+    44985591164829917ull, 45016052289353358ull, 45046534040039159ull, 45077036430853928ull,
+    45107559475773730ull, 45138103188784092ull, 45168667583880014ull, 45199252675065971ull,
+    45229858476355920ull, 45260485001773308ull, 45291132265351078ull, 45321800281131675ull,
+    45352489063167053ull, 45383198625518680ull, 45413928982257545ull, 45444680147464168ull,
+    45475452135228599ull, 45506244959650432ull, 45537058634838808ull, 45567893174912419ull,
+    45598748593999522ull, 45629624906237935ull, 45660522125775054ull, 45691440266767852ull,
+    45722379343382888ull, 45753339369796316ull, 45784320360193886ull, 45815322328770956ull,
+    45846345289732496ull, 45877389257293092ull, 45908454245676958ull, 45939540269117938ull,
+    45970647341859516ull, 46001775478154818ull, 46032924692266624ull, 46064094998467370ull,
+    46095286411039156ull, 46126498944273756ull, 46157732612472616ull, 46188987429946871ull,
+    46220263411017345ull, 46251560570014556ull, 46282878921278731ull, 46314218479159803ull,
+    46345579258017423ull, 46376961272220966ull, 46408364536149536ull, 46439789064191976ull,
+    46471234870746867ull, 46502701970222545ull, 46534190377037101ull, 46565700105618385ull,
+    46597231170404023ull, 46628783585841412ull, 46660357366387734ull, 46691952526509960ull,
+    46723569080684857ull, 46755207043398995ull, 46786866429148753ull, 46818547252440325ull,
+    46850249527789730ull, 46881973269722814ull, 46913718492775260ull, 46945485211492593ull,
+    46977273440430187ull, 47009083194153273ull, 47040914487236944ull, 47072767334266162ull,
+    47104641749835765ull, 47136537748550474ull, 47168455345024899ull, 47200394553883545ull,
+    47232355389760821ull, 47264337867301047ull, 47296342001158455ull, 47328367805997202ull,
+    47360415296491377ull, 47392484487325001ull, 47424575393192039ull, 47456688028796409ull,
+    47488822408851982ull, 47520978548082593ull, 47553156461222048ull, 47585356163014128ull,
+    47617577668212599ull, 47649820991581217ull, 47682086147893734ull, 47714373151933907ull,
+    47746682018495503ull, 47779012762382306ull, 47811365398408124ull, 47843739941396797ull,
+    47876136406182201ull, 47908554807608259ull, 47940995160528942ull, 47973457479808282ull,
+    48005941780320374ull, 48038448076949386ull, 48070976384589563ull, 48103526718145236ull,
+    48136099092530830ull, 48168693522670866ull, 48201310023499973ull, 48233948609962892ull,
+    48266609297014483ull, 48299292099619734ull, 48331997032753764ull, 48364724111401833ull,
+    48397473350559350ull, 48430244765231875ull, 48463038370435129ull, 48495854181195004ull,
+    48528692212547561ull, 48561552479539047ull, 48594434997225896ull, 48627339780674736ull,
+    48660266844962397ull, 48693216205175920ull, 48726187876412561ull, 48759181873779798ull,
+    48792198212395339ull, 48825236907387129ull, 48858297973893357ull, 48891381427062462ull,
+    48924487282053141ull, 48957615554034353ull, 48990766258185333ull, 49023939409695590ull,
+    49057135023764920ull, 49090353115603412ull, 49123593700431453ull, 49156856793479736ull,
+    49190142409989268ull, 49223450565211377ull, 49256781274407716ull, 49290134552850274ull,
+    49323510415821379ull, 49356908878613710ull, 49390329956530299ull, 49423773664884540ull,
+    49457240019000198ull, 49490729034211413ull, 49524240725862708ull, 49557775109308996ull,
+    49591332199915590ull, 49624912013058202ull, 49658514564122961ull, 49692139868506412ull,
+    49725787941615524ull, 49759458798867701ull, 49793152455690785ull, 49826868927523065ull,
+    49860608229813286ull, 49894370378020649ull, 49928155387614828ull, 49961963274075968ull,
+    49995794052894699ull, 50029647739572138ull, 50063524349619901ull, 50097423898560103ull,
+    50131346401925374ull, 50165291875258860ull, 50199260334114230ull, 50233251794055687ull,
+    50267266270657973ull, 50301303779506374ull, 50335364336196733ull, 50369447956335449ull,
+    50403554655539493ull, 50437684449436406ull, 50471837353664315ull, 50506013383871934ull,
+    50540212555718574ull, 50574434884874149ull, 50608680387019183ull, 50642949077844819ull,
+    50677240973052824ull, 50711556088355598ull, 50745894439476180ull, 50780256042148255ull,
+    50814640912116162ull, 50849049065134901ull, 50883480516970141ull, 50917935283398225ull,
+    50952413380206181ull, 50986914823191723ull, 51021439628163266ull, 51055987810939928ull,
+    51090559387351537ull, 51125154373238642ull, 51159772784452518ull, 51194414636855171ull,
+    51229079946319351ull, 51263768728728554ull, 51298480999977032ull, 51333216775969798ull,
+    51367976072622636ull, 51402758905862107ull, 51437565291625556ull, 51472395245861120ull,
+    51507248784527736ull, 51542125923595144ull, 51577026679043901ull, 51611951066865384ull,
+    51646899103061798ull, 51681870803646182ull, 51716866184642421ull, 51751885262085248ull,
+    51786928052020254ull, 51821994570503897ull, 51857084833603503ull, 51892198857397282ull,
+    51927336657974328ull, 51962498251434632ull, 51997683653889086ull, 52032892881459489ull,
+    52068125950278559ull, 52103382876489937ull, 52138663676248197ull, 52173968365718848ull,
+    52209296961078350ull, 52244649478514112ull, 52280025934224507ull, 52315426344418876ull,
+    52350850725317534ull, 52386299093151782ull, 52421771464163909ull, 52457267854607204ull,
+    52492788280745962ull, 52528332758855489ull, 52563901305222113ull, 52599493936143190ull,
+    52635110667927110ull, 52670751516893308ull, 52706416499372268ull, 52742105631705532ull,
+    52777818930245707ull, 52813556411356475ull, 52849318091412596ull, 52885103986799919ull,
+    52920914113915387ull, 52956748489167048ull, 52992607128974058ull, 53028490049766693ull,
+    53064397267986354ull, 53100328800085574ull, 53136284662528028ull, 53172264871788537ull,
+    53208269444353079ull, 53244298396718795ull, 53280351745393997ull, 53316429506898175ull,
+    53352531697762005ull, 53388658334527355ull, 53424809433747296ull, 53460985011986108ull,
+    53497185085819284ull, 53533409671833544ull, 53569658786626838ull, 53605932446808355ull,
+    53642230668998530ull, 53678553469829055ull, 53714900865942879ull, 53751272873994226ull,
+    53787669510648593ull, 53824090792582762ull, 53860536736484810ull, 53897007359054112ull,
+    53933502677001351ull, 53970022707048525ull, 54006567465928956ull, 54043136970387295ull,
+    54079731237179534ull, 54116350283073007ull, 54152994124846406ull, 54189662779289782ull,
+    54226356263204555ull, 54263074593403521ull, 54299817786710864ull, 54336585859962157ull,
+    54373378830004372ull, 54410196713695893ull, 54447039527906514ull, 54483907289517457ull,
+    54520800015421371ull, 54557717722522346ull, 54594660427735916ull, 54631628147989071ull,
+    54668620900220262ull, 54705638701379411ull, 54742681568427913ull, 54779749518338654ull,
+    54816842568096008ull, 54853960734695852ull, 54891104035145571ull, 54928272486464067ull,
+    54965466105681764ull, 55002684909840620ull, 55039928915994130ull, 55077198141207341ull,
+    55114492602556849ull, 55151812317130819ull, 55189157302028984ull, 55226527574362655ull,
+    55263923151254731ull, 55301344049839706ull, 55338790287263675ull, 55376261880684344ull,
+    55413758847271036ull, 55451281204204700ull, 55488828968677921ull, 55526402157894922ull,
+    55564000789071579ull, 55601624879435422ull, 55639274446225650ull, 55676949506693132ull,
+    55714650078100420ull, 55752376177721754ull, 55790127822843070ull, 55827905030762013ull,
+    55865707818787935ull, 55903536204241914ull, 55941390204456752ull, 55979269836776992ull,
+    56017175118558917ull, 56055106067170566ull, 56093062699991738ull, 56131045034413998ull,
+    56169053087840689ull, 56207086877686940ull, 56245146421379669ull, 56283231736357597ull,
+    56321342840071251ull, 56359479749982976ull, 56397642483566941ull, 56435831058309148ull,
+    56474045491707436ull, 56512285801271497ull, 56550552004522876ull, 56588844118994984ull,
+    56627162162233103ull, 56665506151794397ull, 56703876105247917ull, 56742272040174612ull,
+    56780693974167336ull, 56819141924830852ull, 56857615909781849ull, 56896115946648940ull,
+    56934642053072678ull, 56973194246705560ull, 57011772545212036ull, 57050376966268517ull,
+    57089007527563383ull, 57127664246796993ull, 57166347141681689ull, 57205056229941807ull,
+    57243791529313688ull, 57282553057545678ull, 57321340832398144ull, 57360154871643479ull,
+    57398995193066108ull, 57437861814462502ull, 57476754753641178ull, 57515674028422716ull,
+    57554619656639761ull, 57593591656137032ull, 57632590044771333ull, 57671614840411558ull,
+    57710666060938702ull, 57749743724245866ull, 57788847848238269ull, 57827978450833253ull,
+    57867135549960292ull, 57906319163561002ull, 57945529309589145ull, 57984766006010644ull,
+    58024029270803585ull, 58063319121958227ull, 58102635577477011ull, 58141978655374570ull,
+    58181348373677733ull, 58220744750425537ull, 58260167803669232ull, 58299617551472293ull,
+    58339094011910425ull, 58378597203071573ull, 58418127143055931ull, 58457683849975947ull,
+    58497267341956335ull, 58536877637134082ull, 58576514753658455ull, 58616178709691011ull,
+    58655869523405606ull, 58695587212988399ull, 58735331796637867ull, 58775103292564806ull,
+    58814901718992348ull, 58854727094155958ull, 58894579436303456ull, 58934458763695011ull,
+    58974365094603163ull, 59014298447312820ull, 59054258840121274ull, 59094246291338205ull,
+    59134260819285693ull, 59174302442298222ull, 59214371178722694ull, 59254467046918431ull,
+    59294590065257188ull, 59334740252123161ull, 59374917625912994ull, 59415122205035786ull,
+    59455354007913104ull, 59495613052978988ull, 59535899358679960ull, 59576212943475031ull,
+    59616553825835715ull, 59656922024246031ull, 59697317557202515ull, 59737740443214226ull,
+    59778190700802757ull, 59818668348502245ull, 59859173404859373ull, 59899705888433384ull,
+    59940265817796090ull, 59980853211531876ull, 60021468088237712ull, 60062110466523161ull,
+    60102780365010386ull, 60143477802334160ull, 60184202797141876ull, 60224955368093550ull,
+    60265735533861838ull, 60306543313132036ull, 60347378724602093ull, 60388241786982621ull,
+    60429132518996899ull, 60470050939380886ull, 60510997066883227ull, 60551970920265262ull,
+    60592972518301035ull, 60634001879777303ull, 60675059023493543ull, 60716143968261963ull,
+    60757256732907509ull, 60798397336267874ull, 60839565797193504ull, 60880762134547614ull,
+    60921986367206189ull, 60963238514057994ull, 61004518594004588ull, 61045826625960325ull,
+    61087162628852371ull, 61128526621620703ull, 61169918623218126ull, 61211338652610278ull,
+    61252786728775640ull, 61294262870705541ull, 61335767097404174ull, 61377299427888596ull,
+    61418859881188743ull, 61460448476347438ull, 61502065232420396ull, 61543710168476237ull,
+    61585383303596492ull, 61627084656875614ull, 61668814247420983ull, 61710572094352920ull,
+    61752358216804690ull, 61794172633922517ull, 61836015364865587ull, 61877886428806061ull,
+    61919785844929079ull, 61961713632432777ull, 62003669810528285ull, 62045654398439745ull,
+    62087667415404317ull, 62129708880672183ull, 62171778813506563ull, 62213877233183721ull,
+    62256004158992972ull, 62298159610236693ull, 62340343606230331ull, 62382556166302413ull,
+    62424797309794552ull, 62467067056061460ull, 62509365424470953ull, 62551692434403964ull,
+    62594048105254545ull, 62636432456429885ull, 62678845507350311ull, 62721287277449303ull,
+    62763757786173496ull, 62806257052982697ull, 62848785097349886ull, 62891341938761234ull,
+    62933927596716100ull, 62976542090727052ull, 63019185440319869ull, 63061857665033550ull,
+    63104558784420326ull, 63147288818045667ull, 63190047785488292ull, 63232835706340176ull,
+    63275652600206561ull, 63318498486705965ull, 63361373385470189ull, 63404277316144329ull,
+    63447210298386781ull, 63490172351869255ull, 63533163496276778ull, 63576183751307710ull,
+    63619233136673747ull, 63662311672099933ull, 63705419377324669ull, 63748556272099720ull,
+    63791722376190226ull, 63834917709374712ull, 63878142291445095ull, 63921396142206693ull,
+    63964679281478234ull, 64007991729091869ull, 64051333504893175ull, 64094704628741167ull,
+    64138105120508310ull, 64181535000080523ull, 64224994287357190ull, 64268483002251171ull,
+    64312001164688809ull, 64355548794609939ull, 64399125911967899ull, 64442732536729537ull,
+    64486368688875223ull, 64530034388398853ull, 64573729655307866ull, 64617454509623244ull,
+    64661208971379529ull, 64704993060624827ull, 64748806797420822ull, 64792650201842779ull,
+    64836523293979559ull, 64880426093933624ull, 64924358621821050ull, 64968320897771533ull,
+    65012312941928398ull, 65056334774448613ull, 65100386415502792ull, 65144467885275209ull,
+    65188579203963805ull, 65232720391780196ull, 65276891468949686ull, 65321092455711273ull,
+    65365323372317660ull, 65409584239035264ull, 65453875076144225ull, 65498195903938413ull,
+    65542546742725443ull, 65586927612826678ull, 65631338534577245ull, 65675779528326036ull,
+    65720250614435724ull, 65764751813282772ull, 65809283145257437ull, 65853844630763785ull,
+    65898436290219698ull, 65943058144056884ull, 65987710212720884ull, 66032392516671086ull,
+    66077105076380729ull, 66121847912336917ull, 66166621045040626ull, 66211424495006714ull,
+    66256258282763928ull, 66301122428854920ull, 66346016953836248ull, 66390941878278391ull,
+    66435897222765758ull, 66480883007896694ull, 66525899254283495ull, 66570945982552411ull,
+    66616023213343659ull, 66661130967311435ull, 66706269265123918ull, 66751438127463282ull,
+    66796637575025708ull, 66841867628521387ull, 66887128308674537ull, 66932419636223408ull,
+    66977741631920293ull, 67023094316531534ull, 67068477710837539ull, 67113891835632784ull,
+    67159336711725826ull, 67204812359939314ull, 67250318801109994ull, 67295856056088723ull,
+    67341424145740476ull, 67387023090944357ull, 67432652912593607ull, 67478313631595614ull,
+    67524005268871926ull, 67569727845358253ull, 67615481382004486ull, 67661265899774698ull,
+    67707081419647159ull, 67752927962614345ull, 67798805549682945ull, 67844714201873873ull,
+    67890653940222277ull, 67936624785777548ull, 67982626759603331ull, 68028659882777532ull,
+    68074724176392333ull, 68120819661554194ull, 68166946359383871ull, 68213104291016418ull,
+    68259293477601201ull, 68305513940301909ull, 68351765700296559ull, 68398048778777511ull,
+    68444363196951471ull, 68490708976039508ull, 68537086137277060ull, 68583494701913943ull,
+    68629934691214362ull, 68676406126456923ull, 68722909028934637ull, 68769443419954936ull,
+    68816009320839678ull, 68862606752925159ull, 68909235737562123ull, 68955896296115771ull,
+    69002588449965772ull, 69049312220506270ull, 69096067629145897ull, 69142854697307780ull,
+    69189673446429555ull, 69236523897963370ull, 69283406073375904ull, 69330319994148366ull,
+    69377265681776516ull, 69424243157770667ull, 69471252443655695ull, 69518293560971055ull,
+    69565366531270786ull, 69612471376123521ull, 69659608117112497ull, 69706776775835568ull,
+    69753977373905212ull, 69801209932948539ull, 69848474474607307ull, 69895771020537925ull,
+    69943099592411470ull, 69990460211913688ull, 70037852900745015ull, 70085277680620576ull,
+    70132734573270202ull, 70180223600438440ull, 70227744783884557ull, 70275298145382555ull,
+    70322883706721183ull, 70370501489703940ull, 70418151516149090ull, 70465833807889672ull,
+    70513548386773507ull, 70561295274663211ull, 70609074493436204ull, 70656886064984718ull,
+    70704730011215812ull, 70752606354051376ull, 70800515115428146ull, 70848456317297711ull,
+    70896429981626524ull, 70944436130395913ull, 70992474785602090ull, 71040545969256161ull,
+    71088649703384136ull, 71136786010026940ull, 71184954911240422ull, 71233156429095368ull,
+    71281390585677505ull, 71329657403087519ull, 71377956903441057ull, 71426289108868745ull,
+    71474654041516191ull, 71523051723544001ull, 71571482177127785ull, 71619945424458170ull,
+    71668441487740808ull, 71716970389196388ull, 71765532151060644ull, 71814126795584367ull,
+    71862754345033417ull, 71911414821688726ull, 71960108247846319ull, 72008834645817313ull,
 };
 
 }  // namespace gen

@@ -15,8 +15,6 @@
 namespace lbm39 {
 namespace {
 
-constexpr int BLK = 64;  // the step kernel's block (the workspace is laid out per block)
-constexpr size_t WS_BYTES = (size_t)BLK * WS_DOUBLES * sizeof(double);
 
 // f_i of the current state in FP64 (the stored deviation plus h_ref in the
 // precision form; exact).
@@ -48,10 +46,12 @@ __device__ __forceinline__ Macro moments_at(const Desc& d, long long cell, bool 
 // the solve fails (the cell takes the fallback equilibrium).  Non-fluid cells
 // read 0.  odd: the AA parity of the lattice's time.
 template <class P, bool D2, int SOLVER = 0>
-__global__ void __launch_bounds__(BLK) k_diag_fields(Desc d, int odd, double* eps_out,
-                                                     int* nupd_out) {
+__global__ void __launch_bounds__(solve_blk(in_fixed_point<P, SOLVER>))
+    k_diag_fields(Desc d, int odd, double* eps_out, int* nupd_out) {
+  constexpr bool FIXED = in_fixed_point<P, SOLVER>;
+  constexpr int BLK = solve_blk(FIXED);
   extern __shared__ double smem[];
-  load_exp_table();
+  load_solver_table<FIXED>();
   const long long cell = (long long)blockIdx.x * BLK + threadIdx.x;
   if (cell >= d.N) return;
   if (d.mask != nullptr && d.mask[cell] != MASK_FLUID) {
@@ -67,8 +67,11 @@ __global__ void __launch_bounds__(BLK) k_diag_fields(Desc d, int odd, double* ep
   const bool marked = is_fallback_embedding<BLK>(lam);
   const int maxit = !marked ? d.ph.maxit : retry_budget(d.t, d.ph.maxit);
   int n32;
-  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(w, d.ph, maxit, n32);
-  if (nr.failed) fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);
+  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32);
+  if (nr.failed) {
+    targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // the solve may have overwritten them
+    fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);
+  }
   double f[Q];
   if (odd) gather_f<true, P>(d, cell, f);
   else gather_f<false, P>(d, cell, f);
@@ -82,6 +85,14 @@ __global__ void __launch_bounds__(BLK) k_diag_fields(Desc d, int odd, double* ep
   nupd_out[cell] = nr.failed ? -1 : nr.n_upd;
 }
 
+template <class P, bool D2, int SOLVER = 0>
+void launch_diag(const LatticeView& v, int odd, double* eps, int* n_upd) {
+  constexpr bool FIXED = in_fixed_point<P, SOLVER>;
+  constexpr int BLK = solve_blk(FIXED);
+  launch_ws<k_diag_fields<P, D2, SOLVER>>((unsigned)((v.N + BLK - 1) / BLK), BLK,
+                                          ws_bytes(FIXED), v.stream, v.desc, odd, eps, n_upd);
+}
+
 }  // namespace
 }  // namespace lbm39
 
@@ -90,25 +101,24 @@ extern "C" int lbm39_diag_fields(lbm39_lattice* L, double* eps, int32_t* n_upd) 
   LatticeView v;
   if (!lattice_view(L, &v) || !eps || !n_upd) return LBM39_ERR_ARG;
   if (!v.initialized) return LBM39_ERR_STATE;
-  const unsigned grid = (unsigned)((v.N + BLK - 1) / BLK);
   const int odd = (int)(v.desc.t & 1);
   if (v.mixed)
-    k_diag_fields<float, false><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<float, false>(v, odd, eps, n_upd);
   else if (v.solver == 1 && v.desc.d2)
-    k_diag_fields<double, true, 1><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, true, 1>(v, odd, eps, n_upd);
   else if (v.solver == 1)
-    k_diag_fields<double, false, 1><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, false, 1>(v, odd, eps, n_upd);
   else if (v.solver == 2 && v.desc.d2)
-    k_diag_fields<double, true, 2><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, true, 2>(v, odd, eps, n_upd);
   else if (v.solver == 2)
-    k_diag_fields<double, false, 2><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, false, 2>(v, odd, eps, n_upd);
   else if (v.solver == 3 && v.desc.d2)
-    k_diag_fields<double, true, 3><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, true, 3>(v, odd, eps, n_upd);
   else if (v.solver == 3)
-    k_diag_fields<double, false, 3><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, false, 3>(v, odd, eps, n_upd);
   else if (v.desc.d2)
-    k_diag_fields<double, true><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, true>(v, odd, eps, n_upd);
   else
-    k_diag_fields<double, false><<<grid, BLK, WS_BYTES, v.stream>>>(v.desc, odd, eps, n_upd);
+    launch_diag<double, false>(v, odd, eps, n_upd);
   return cudaGetLastError() == cudaSuccess ? LBM39_OK : LBM39_ERR_CUDA;
 }

@@ -14,8 +14,9 @@
 
 namespace lbm39 {
 
-// Per-block copy of the table in shared memory; every kernel that evaluates
-// equilibria first runs load_exp_table() with the whole block.
+// Per-block copy of the table in shared memory, for the kernels whose solves are
+// all in FP64; they first run load_exp_table() with the whole block.  The others
+// read the few values they need from the table in device memory.
 __device__ __forceinline__ double* exp_table() {
   __shared__ double t[256];
   return t;
@@ -32,7 +33,7 @@ __device__ __forceinline__ int exp_out_of_range(double x) {
   return (__double2hiint(x) & 0x7ff00000) >= ((1023 + 9) << 20);
 }
 
-__device__ __forceinline__ double exp_tang_core(double x) {
+__device__ __forceinline__ double exp_tang_core(double x, const double* __restrict__ tab) {
   const double shifter = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer in the low word
   const double t = fma(x, gen::EXP_INV_L, shifter);
   const int k = __double2loint(t);
@@ -42,14 +43,14 @@ __device__ __forceinline__ double exp_tang_core(double x) {
   double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
   q = fma(q, r, 0.5);
   q = fma(q, r, 1.0);
-  const double T = exp_table()[k & 255];
+  const double T = tab[k & 255];
   const double y = fma(T * r, q, T);
   const int scale = (int)((unsigned)(k >> 8) << 20);  // 2^m in the exponent field
   return __hiloint2double(__double2hiint(y) + scale, __double2loint(y));
 }
 
 __device__ __forceinline__ double exp_tang(double x) {
-  return exp_out_of_range(x) ? exp(x) : exp_tang_core(x);
+  return exp_out_of_range(x) ? exp(x) : exp_tang_core(x, exp_table());
 }
 
 }  // namespace lbm39

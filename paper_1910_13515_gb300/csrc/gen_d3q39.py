@@ -18,6 +18,9 @@ Emitted:
   moments<T>(F, s, J)         s_k = sum_i F_i phi_k,  J_kl = sum_i F_i phi_k phi_l (packed)
   f_moments(f, ...)           rho, j, sum f|xi|^2;  g_sum(g): sum g
   exp2_table                  2^(j/256), j = 0..255, correctly rounded (decimal arithmetic)
+  sums_fx, sums_fx2d          sum_i v(i) phi_k(xi_i) in 64-bit integers, orbit by orbit
+  jvec_fx, jvec_fx2d          sum_i p(i, y_i) phi_k(xi_i) with y_i = sum_k d_k phi_k(xi_i)
+  exp2_fixed                  2^(j/1024) 2^55, j = 0..1023, nearest integers
   exp constants               ln2/256 split in a 32-bit head and a tail
 """
 from __future__ import annotations
@@ -419,6 +422,145 @@ def exp_constants():
     return float(inv), float(L_hi), float(L_lo), [float(t) for t in table]
 
 
+# The integer forms: each orbit's values are read, folded and added to the results before the next
+# orbit is touched, so that few registers are live.  Integer sums are exact, so their order does
+# not matter, and the z-mirror form (basis functions even in xi_z, values equal under the mirror)
+# reads one velocity of each mirror pair and counts it twice with the same result.
+
+def _orbit_terms(ks):
+    """Per orbit: {sign subset T: [(result index, integer factor)]} of the basis functions ks."""
+    out = []
+    for key, axes, members in ORBITS:
+        use = {}
+        for pos, k in enumerate(ks):
+            p, m = GBASIS[k]
+            if any(p[a] != 0 and key[a] == 0 for a in range(3)):
+                continue
+            mag = sum(c * c for c in key) ** m
+            for a in range(3):
+                mag *= key[a] ** p[a]
+            if mag:
+                use.setdefault(tuple(a for a in axes if p[a] % 2 == 1), []).append((pos, mag))
+        out.append(use)
+    return out
+
+
+def gen_int_sums(zsym=False, jvec=False):
+    em = Emitter()
+    ks = ZEVEN if zsym else list(range(NM))
+    n = len(ks)
+    name = ("jvec_fx" if jvec else "sums_fx") + ("2d" if zsym else "")
+    em(f"// s_k = sum_i {'p(i, y_i)' if jvec else 'v(i)'} phi_k(xi_i) in 64-bit integers"
+       + (" (the nine z-even k, values mirror-symmetric in z)." if zsym else "."))
+    em("template <class V>")
+    if jvec:
+        em(f"__device__ __forceinline__ void {name}(const int (&d)[{n}], const V& p, "
+           f"unsigned long long (&s)[{n}]) {{")
+    else:
+        em(f"__device__ __forceinline__ void {name}(const V& v, unsigned long long (&s)[{n}]) {{")
+    first = [True] * n
+    for o, ((key, axes, members), use) in enumerate(zip(ORBITS, _orbit_terms(ks))):
+        # a z-mirror pair enters once: fold over the other axes only
+        ax = [a for a in axes if not (zsym and a == 2)]
+        double = 2 if zsym and 2 in axes else 1
+        mem = {}
+        for sg, i in members.items():
+            sd = dict(zip(axes, sg))
+            if zsym and 2 in axes and sd[2] < 0:
+                continue
+            mem[tuple(sd[a] for a in ax)] = i
+        cur = {}
+        if jvec:  # y of the orbit's members: coefficients of the sign subsets, then butterflies
+            cT = {}
+            for T in subsets(ax):
+                terms = []
+                for pos, k in enumerate(ks):
+                    coef = 0
+                    for pw, c in BASIS[k].items():
+                        if any(pw[a] != 0 and key[a] == 0 for a in range(3)):
+                            continue
+                        if tuple(a for a in axes if pw[a] % 2 == 1) != T:
+                            continue
+                        for a in range(3):
+                            c *= key[a] ** pw[a]
+                        coef += c
+                    if coef:
+                        terms.append((coef, f"d[{pos}]"))
+                if terms:
+                    nm = f"c{o}_{''.join('xyz'[a] for a in T) or '0'}"
+                    em(f"  const int {nm} = "
+                       + " + ".join(v if c == 1 else f"{c} * {v}" for c, v in terms) + ";")
+                    cT[T] = nm
+            vals = {((), T): v for T, v in cT.items()}
+            for j, a in enumerate(ax):
+                nxt = {}
+                keys = sorted({(sg, tuple(t for t in T if t != a)) for sg, T in vals})
+                for sg, T in keys:
+                    e, w = vals.get((sg, T)), vals.get((sg, tuple(sorted(T + (a,)))))
+                    for sa in (1, -1):
+                        if w is None:
+                            nxt[(sg + (sa,), T)] = e
+                            continue
+                        nm = f"y{o}_{j}_{len(nxt)}"
+                        em(f"  const int {nm} = "
+                           + (f"{e} {'+' if sa == 1 else '-'} {w};" if e
+                              else f"{'' if sa == 1 else '-'}{w};"))
+                        nxt[(sg + (sa,), T)] = nm
+                vals = nxt
+            for sg, i in mem.items():
+                em(f"  const unsigned long long p{i} = p(Idx<{i}>{{}}, {vals[(sg, ())]});")
+                cur[sg] = f"p{i}"
+        else:
+            for sg, i in mem.items():
+                em(f"  const unsigned long long v{i} = v(Idx<{i}>{{}});")
+                cur[sg] = f"v{i}"
+        need = set(use)
+        for stage, a in enumerate(ax):
+            nxt = {}
+            for sg in sorted((x for x in cur if x[stage] == 1), key=str):
+                sm = sg[:stage] + (-1,) + sg[stage + 1:]
+                for tag, op in (("E", "+"), ("O", "-")):
+                    nk = sg[:stage] + (tag,) + sg[stage + 1:]
+                    nm = f"w{o}_{stage}_{len(nxt)}"
+                    em(f"  const unsigned long long {nm} = {cur[sg]} {op} {cur[sm]};")
+                    nxt[nk] = nm
+            cur = nxt
+        for sg, v in cur.items():
+            T = tuple(a for a, t in zip(ax, sg) if t == "O")
+            for pos, mag in use.get(T, []):
+                c = mag * double
+                term = v if c == 1 else f"{c}ull * {v}"
+                em(f"  s[{pos}] {'=' if first[pos] else '+='} {term};")
+                first[pos] = False
+        assert need <= {tuple(a for a, t in zip(ax, sg) if t == "O") for sg in cur}
+    em("}")
+    return em.lines
+
+
+def selfcheck_int(lines, zsym, jvec):
+    """The emitted integer sums against direct sums over the 39 velocities."""
+    import random
+    import re
+    rnd = random.Random(5)
+    ks = ZEVEN if zsym else list(range(NM))
+    F = [rnd.randrange(1, 1 << 20) for _ in range(Q)]
+    if zsym:
+        for i in range(Q):
+            F[i] = F[VEL.index((VEL[i][0], VEL[i][1], abs(VEL[i][2])))]
+    d = [rnd.randrange(-1 << 20, 1 << 20) for _ in ks]
+    y = [sum(c * phi(k, v) for c, k in zip(d, ks)) for v in VEL]
+    env = {"v": lambda i: F[i], "p": lambda i, t: F[i] * t, "d": d, "s": [None] * len(ks)}
+    for ln in lines[3:-1]:
+        t = re.sub(r"Idx<(\d+)>\{\}", r"\1", ln.strip())
+        t = t.replace("ull", "")
+        t = re.sub(r"^const (int|unsigned long long) ", "", t).rstrip(";")
+        # `p` and `v` are both functions and prefixes of names: names carry a digit
+        exec(t, env)
+    for pos, k in enumerate(ks):
+        ref = sum((F[i] * y[i] if jvec else F[i]) * phi(k, VEL[i]) for i in range(Q))
+        assert env["s"][pos] == ref, (zsym, jvec, k)
+
+
 def selfcheck(lines):
     """Evaluate the emitted straight-line code in Python on random inputs and compare with
     the direct sums over the 39 velocities."""
@@ -569,13 +711,30 @@ def generate():
     lines.append(f"constexpr double EXP_L_HI = {L_hi!r};")
     lines.append(f"constexpr double EXP_L_LO = {L_lo!r};")
     lines.append("// 2^(j/256), j = 0..255, each the double nearest the exact value.")
-    lines.append("__device__ __constant__ double kExp2Table[256] = {")
+    lines.append("__device__ const double kExp2Table[256] = {")
     for j in range(0, 256, 4):
         lines.append("    " + ", ".join(repr(t) for t in table[j:j + 4]) + ",")
     lines.append("};")
-    lines += ["", "}  // namespace gen", "}  // namespace lbm39", ""]
     selfcheck(strip_2d(lines))
     selfcheck_2d(lines)
+    lines += ["", "// A velocity index as a type.", "template <int I>", "struct Idx {",
+              "  static constexpr int value = I;", "};"]
+    int_lines = []
+    for zsym in (False, True):
+        for jvec in (False, True):
+            body = gen_int_sums(zsym, jvec)
+            selfcheck_int(body, zsym, jvec)
+            int_lines += [""] + body
+    lines += int_lines
+    lines.append("")
+    lines.append("// 2^(j/1024) in units of 2^-55, j = 0..1023, each the integer nearest the exact value.")
+    lines.append("__device__ const unsigned long long kExp2Fixed[1024] = {")
+    tab = [int((D(2) ** (D(j) / 1024 + 55)).to_integral_value(rounding=decimal.ROUND_HALF_EVEN))
+           for j in range(1024)]
+    for j in range(0, 1024, 4):
+        lines.append("    " + ", ".join(f"{t}ull" for t in tab[j:j + 4]) + ",")
+    lines.append("};")
+    lines += ["", "}  // namespace gen", "}  // namespace lbm39", ""]
     return lines, nmono
 
 

@@ -25,6 +25,8 @@
 #include <cstdint>
 
 #include "cell.cuh"
+#include "launch.cuh"
+#include "solve_fx.cuh"
 
 namespace lbm39 {
 
@@ -376,7 +378,9 @@ __device__ __forceinline__ void store_solver_state(const Desc& d, long long cell
 template <int BLK>
 __device__ __forceinline__ void eval_at_lam(WS<BLK> w) {
   double G[NM];
-  eval_equilibrium<BLK>(w.at(WS_LAM), w.at(WS_DL), 0.0, w.at(WS_E), w.at(WS_M), G, false);
+  const WS<1> none{nullptr};
+  eval_equilibrium<BLK>(w.at(WS_LAM), none, 0.0, w.at(WS_E), w.at(WS_M), G, false,
+                        gen::kExp2Table);
 }
 
 // Where the 13-moment solve failed or took no update: the fallback's
@@ -418,27 +422,60 @@ __device__ __forceinline__ int retry_budget(long long t, int maxit) {
   return (t & (RETRY_PERIOD - 1)) == 0 ? maxit : 0;
 }
 
+// Whether a kernel solves in fixed point.  The chord-Newton hybrid does not: its factor fills the
+// registers.  Nor does the precision form: its stores round F to FP32 deviations, and a last bit
+// of F that falls the other way there changes the stored state by 1e-9 and grows with the flow.
+template <class P, int SOLVER>
+constexpr bool in_fixed_point = sizeof(P) == 8 && SOLVER != 1;
+
+// Threads per block of the kernels that solve, and their workspace (the FP64 solves keep their
+// direction there too).
+constexpr int solve_blk(bool fixed) { return fixed ? 128 : 64; }
+constexpr int solve_min_blocks(bool fixed) { return fixed ? 3 : 4; }
+constexpr size_t ws_bytes(bool fixed) {
+  return (size_t)solve_blk(fixed) * (fixed ? WS_DOUBLES_FX : WS_DOUBLES) * sizeof(double);
+}
+
+// The table of the exponential that the solver reads, for the whole block.
+template <bool FIXED>
+__device__ __forceinline__ void load_solver_table() {
+  if constexpr (FIXED) fx::load_table();
+  else load_exp_table();
+}
+
 // The constraint solve of a cell from the warm start in the workspace (F cached
 // at lam) with the lattice's root finder SOLVER (FP64 path): 0 Newton-Raphson;
 // 1 the chord-Newton hybrid (newton_chord); 2 Newton with a single-precision
-// direction (newton<BLK, true>); 3 that after a single-precision start
-// (start32).  The precision form (P = float) always takes 3.  n32: the float
-// steps of the start.
+// direction; 3 that after a single-precision start (start32).  The precision
+// form (P = float) always takes 3.  n32: the float steps of the start.
+// In fixed point (newton_fx) where in_fixed_point says so; a cell that it cannot
+// represent is solved again from the stored state in FP64 (newton).
 template <class P, int BLK, bool D2, int SOLVER>
-__device__ __forceinline__ NewtonResult solve_cell(WS<BLK> w, const Phys& ph, int maxit,
-                                                   int& n32) {
+__device__ __forceinline__ NewtonResult solve_cell(const Desc& d, long long cell, WS<BLK> w,
+                                                   const Macro& M, int maxit, int& n32) {
+  constexpr bool MIXED = sizeof(P) == 4 || SOLVER >= 2, START = sizeof(P) == 4 || SOLVER == 3;
   n32 = 0;
-  if constexpr (SOLVER == 1 && sizeof(P) == 8) {
-    return newton_chord<BLK, D2>(w, ph, maxit, true);
-  } else {
-    bool cached = true;
-    if constexpr (sizeof(P) == 4 || SOLVER == 3) {
-      if (maxit > 0) {  // a cell on the fallback off a retry step takes no step at all
-        n32 = start32<BLK, D2>(w);
-        cached = n32 == 0;
-      }
+  bool cached = true;
+  if constexpr (START) {
+    if (maxit > 0) {  // a cell on the fallback off a retry step takes no step at all
+      n32 = start32<BLK, D2>(w);
+      cached = n32 == 0;
     }
-    return newton<BLK, sizeof(P) == 4 || SOLVER >= 2, D2>(w, ph, maxit, cached);
+  }
+  if constexpr (SOLVER == 1 && sizeof(P) == 8) {
+    return newton_chord<BLK, D2>(w, d.ph, maxit, true);
+  } else if constexpr (!in_fixed_point<P, SOLVER>) {
+    return newton_in<BLK, MIXED, D2>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd, maxit,
+                                     cached);
+  } else {
+    NewtonResult nr;
+    if (d.ph.fx && newton_fx<BLK, !MIXED, D2>(w, d.ph, maxit, cached, nr)) return nr;
+    targets<BLK>(M.ux, M.uy, M.uz, M.T, w.at(WS_M));
+    load_solver_state<BLK>(d, cell, w);
+    if constexpr (START) {
+      if (maxit > 0) start32<BLK, D2>(w);  // as above: the same cached
+    }
+    return newton<BLK, MIXED, D2>(w, d.ph.tol, d.ph.min_upd, maxit, cached);
   }
 }
 
@@ -461,9 +498,11 @@ __device__ __forceinline__ void step_cell(const Desc& d, long long cell, WS<BLK>
   // unless its embedding already meets the 13 constraints)
   const int maxit = !marked ? d.ph.maxit : retry_budget(d.t, d.ph.maxit);
   int n32;
-  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(w, d.ph, maxit, n32);
-  if (nr.failed) fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);
-  else lam[9] = lam[9] + 0.0;  // a solved state carries no embedding mark
+  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32);
+  if (nr.failed) {
+    targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // the solve may have overwritten them
+    fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);
+  } else lam[9] = lam[9] + 0.0;  // a solved state carries no embedding mark
   store_solver_state<BLK>(d, cell, w);
   const int branch = relax_push<ODD, P, BLK, PR>(d, cell, fresh_nbr<ODD>(d, c), M, F);
   atomicAdd(&s_ctr[CTR_FAILED], (unsigned)nr.failed);
@@ -478,11 +517,11 @@ __device__ __forceinline__ void step_cell(const Desc& d, long long cell, WS<BLK>
 
 // One time step over every fluid cell (even or odd AA pass).
 template <bool ODD, class P, int BLK, bool D2, bool PR = false, int SOLVER = 0>
-__global__ void __launch_bounds__(BLK) k_step(Desc d) {
+__global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, SOLVER>)) k_step(Desc d) {
   extern __shared__ double smem[];
   __shared__ unsigned int s_ctr[CTR_N];
   for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
-  load_exp_table();
+  load_solver_table<in_fixed_point<P, SOLVER>>();
   const long long cell = (long long)blockIdx.x * BLK + threadIdx.x;
   if (cell < d.N && (d.mask == nullptr || d.mask[cell] == MASK_FLUID))
     step_cell<ODD, P, BLK, D2, PR, SOLVER>(d, cell, WS<BLK>{smem + threadIdx.x}, s_ctr);
@@ -506,7 +545,7 @@ __global__ void __launch_bounds__(BLK) k_init(Desc d, const double* rho, const d
   extern __shared__ double smem[];
   __shared__ unsigned int s_ctr[CTR_N];
   for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
-  load_exp_table();
+  load_solver_table<in_fixed_point<P, 0>>();
   const long long r = (long long)blockIdx.x * BLK + threadIdx.x;
   const long long cell = c0 + r;
   P* pop = static_cast<P*>(d.pop);
@@ -520,8 +559,19 @@ __global__ void __launch_bounds__(BLK) k_init(Desc d, const double* rho, const d
       WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M);
       targets<BLK>(ux, uy, uz, TT, m);
       gaussian_guess<BLK>(ux, uy, uz, TT, lam);
-      const NewtonResult nr = newton<BLK, false>(w, d.ph, maxit, false);
-      if (nr.failed) fallback_cell<BLK>(d.lam, d.Np, cell, w, TT, false);
+      NewtonResult nr;
+      if constexpr (!in_fixed_point<P, 0>) {
+        nr = newton_in<BLK, false, false>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd,
+                                          maxit, false);
+      } else if (!d.ph.fx || !newton_fx<BLK, true, false>(w, d.ph, maxit, false, nr)) {
+        targets<BLK>(ux, uy, uz, TT, m);
+        gaussian_guess<BLK>(ux, uy, uz, TT, lam);
+        nr = newton<BLK, false>(w, d.ph.tol, d.ph.min_upd, maxit, false);
+      }
+      if (nr.failed) {
+        targets<BLK>(ux, uy, uz, TT, m);
+        fallback_cell<BLK>(d.lam, d.Np, cell, w, TT, false);
+      }
       store_solver_state<BLK>(d, cell, w);
       const double cgr = d.ph.cg * TT * rr;
       for (int i = 0; i < Q; ++i) {
@@ -547,13 +597,12 @@ __global__ void __launch_bounds__(BLK) k_state_equilibrium(Phys ph, double rho, 
                                                            double* out78, int maxit,
                                                            unsigned long long* failed) {
   extern __shared__ double smem[];
-  load_exp_table();
   if (threadIdx.x != 0) return;
   WS<BLK> w{smem};
   WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M);
   targets<BLK>(ux, uy, uz, T, m);
   gaussian_guess<BLK>(ux, uy, uz, T, lam);
-  const NewtonResult nr = newton<BLK, false>(w, ph, maxit, false);
+  const NewtonResult nr = newton<BLK, false>(w, ph.tol, ph.min_upd, maxit, false);
   for (int i = 0; i < Q; ++i) {
     out78[i] = rho * F[i];
     out78[Q + i] = ph.cg * T * rho * F[i];

@@ -27,8 +27,6 @@ using namespace lbm39;
 
 namespace {
 
-constexpr int BLK = 64;                          // threads per block of the cell kernels
-constexpr size_t WS_BYTES = (size_t)BLK * WS_DOUBLES * sizeof(double);
 constexpr int RED_BLOCKS = 1024;                 // blocks of the conserved-sum reduction
 constexpr int RED_THREADS = 128;
 constexpr long long STAGE_CELLS = 1LL << 20;     // host staging chunk (cells)
@@ -167,6 +165,9 @@ static int last_launch() { return cudaGetLastError() == cudaSuccess ? LBM39_OK :
 // Kernel launches for one storage type.
 template <class P>
 struct Launch {
+  static constexpr bool FIXED = in_fixed_point<P, 0>;
+  static constexpr int BLK = solve_blk(FIXED);  // threads per block of the cell kernels
+  static constexpr size_t WSB = ws_bytes(FIXED);
   static void step(lbm39_lattice* L, bool odd) {
     L->desc.t = L->t;
     const unsigned grid = (unsigned)((L->N + BLK - 1) / BLK);
@@ -190,20 +191,20 @@ struct Launch {
       return;
     }
     if (!odd) {
-      if (fp64 && L->desc.d2) k_step<false, P, BLK, fp64><<<grid, BLK, WS_BYTES, L->stream>>>(L->desc);
-      else k_step<false, P, BLK, false><<<grid, BLK, WS_BYTES, L->stream>>>(L->desc);
+      if (fp64 && L->desc.d2) launch_ws<k_step<false, P, BLK, fp64>>(grid, BLK, WSB, L->stream, L->desc);
+      else launch_ws<k_step<false, P, BLK, false>>(grid, BLK, WSB, L->stream, L->desc);
       if (L->fills) k_fill_even<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
     } else {
-      if (fp64 && L->desc.d2) k_step<true, P, BLK, fp64><<<grid, BLK, WS_BYTES, L->stream>>>(L->desc);
-      else k_step<true, P, BLK, false><<<grid, BLK, WS_BYTES, L->stream>>>(L->desc);
+      if (fp64 && L->desc.d2) launch_ws<k_step<true, P, BLK, fp64>>(grid, BLK, WSB, L->stream, L->desc);
+      else launch_ws<k_step<true, P, BLK, false>>(grid, BLK, WSB, L->stream, L->desc);
       if (L->fills) k_fill_odd<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
     }
   }
   static void init(lbm39_lattice* L, const double* rho, const double* u, long long us,
                    const double* T, long long c0, long long len) {
     const unsigned grid = (unsigned)((len + BLK - 1) / BLK);
-    k_init<P, BLK><<<grid, BLK, WS_BYTES, L->stream>>>(L->desc, rho, u, us, T, c0, len,
-                                                       L->p.init_maxit);
+    launch_ws<k_init<P, BLK>>(grid, BLK, WSB, L->stream, L->desc, rho, u, us, T, c0, len,
+                              L->p.init_maxit);
   }
   static void macros(lbm39_lattice* L, double* rho, double* u, long long us, double* T,
                      double* p, long long c0, long long len) {
@@ -298,8 +299,8 @@ static int state_equilibrium(const Phys& ph, cudaStream_t s, double rho, const d
                              double T, int maxit, double* dev78, unsigned long long* dfail,
                              double* host78) {
   CUDA_OK(cudaMemsetAsync(dfail, 0, sizeof(unsigned long long), s));
-  k_state_equilibrium<BLK><<<1, BLK, WS_BYTES, s>>>(ph, rho, u[0], u[1], u[2], T, dev78, maxit,
-                                                     dfail);
+  k_state_equilibrium<32><<<1, 32, 32 * WS_DOUBLES_FX * sizeof(double), s>>>(
+      ph, rho, u[0], u[1], u[2], T, dev78, maxit, dfail);
   if (last_launch() != LBM39_OK) return LBM39_ERR_CUDA;
   unsigned long long nf = 0;
   CUDA_OK(cudaMemcpyAsync(host78, dev78, sizeof(double) * 2 * Q, cudaMemcpyDeviceToHost, s));
@@ -372,6 +373,14 @@ int lbm39_create(const lbm39_params* p, const int32_t* vel, const double* w, voi
   d.ph.tol = p->newton_tol;
   d.ph.maxit = p->newton_maxit;
   d.ph.min_upd = p->newton_min_upd;
+  {
+    // the fixed-point solve resolves residuals to about 1e-16 in units of 2^-58; a tolerance
+    // whose hundredth is nearer to that than a factor of 16, or above its range, stays in FP64
+    const double unit = 0x1p58;
+    d.ph.fx = p->newton_tol >= 2e-13 && p->newton_tol <= 1.0;
+    d.ph.tol_fx = d.ph.fx ? (unsigned long long)std::ceil(p->newton_tol * unit) : 0;
+    d.ph.tol_fx100 = d.ph.fx ? (unsigned long long)std::ceil(1e-2 * p->newton_tol * unit) : 0;
+  }
   d.ph.kn_sensor = p->kn_sensor ? 1 : 0;
   {
     const double alpha[4] = {1.0, 1.05, 1.35, 1.0 / p->tau};  // Eq. (alpha)
@@ -769,7 +778,12 @@ struct BatchLayout {
   long long maxtiles, maxftiles;
 };
 
+// Cells of a tile of the packed step: one block of the step kernel.
+int tile_cells(int precision) { return solve_blk(precision != LBM39_MIXED); }
+
 BatchLayout batch_layout(int maxlat, long long maxcells) {
+  constexpr int BLK = solve_blk(false);  // the smaller tiles: the buffer serves both precisions
+  static_assert(solve_blk(false) <= solve_blk(true), "tiles");
   BatchLayout b;
   b.maxtiles = (maxcells + BLK - 1) / BLK + maxlat;
   b.maxftiles = (maxcells + 255) / 256 + maxlat;
@@ -784,11 +798,13 @@ BatchLayout batch_layout(int maxlat, long long maxcells) {
 template <class P>
 int batch_enqueue(lbm39_batch* B, int s) {
   const int nt = (int)B->hT.size(), nf = (int)B->hF.size(), n2 = B->nT2;
+  constexpr int BLK = Launch<P>::BLK;
+  constexpr size_t WSB = Launch<P>::WSB;
   if constexpr (sizeof(P) == 8) {
-    if (n2) k_batch_step<P, BLK, true><<<n2, BLK, WS_BYTES, B->stream>>>(B->dE, B->dT, s);
+    if (n2) launch_ws<k_batch_step<P, BLK, true>>(n2, BLK, WSB, B->stream, B->dE, B->dT, s);
   }
   if (nt > n2)
-    k_batch_step<P, BLK, false><<<nt - n2, BLK, WS_BYTES, B->stream>>>(B->dE, B->dT + n2, s);
+    launch_ws<k_batch_step<P, BLK, false>>(nt - n2, BLK, WSB, B->stream, B->dE, B->dT + n2, s);
   if (nf) k_batch_fill<P><<<nf, 256, 0, B->stream>>>(B->dE, B->dF, s);
   return last_launch();
 }
@@ -820,16 +836,13 @@ int lbm39_batch_create(int32_t max_lattices, int64_t max_cells, int32_t precisio
     return LBM39_ERR_ARG;
   if (cuda_stream == nullptr) return LBM39_ERR_ARG;  // graphs cannot be captured on the legacy stream
   if (precision != LBM39_FP64 && precision != LBM39_MIXED) return LBM39_ERR_ARG;
-  static bool attr = false;
-  if (!attr) {
-    CUDA_OK(cudaFuncSetAttribute(k_batch_step<double, BLK, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS_BYTES));
-    CUDA_OK(cudaFuncSetAttribute(k_batch_step<double, BLK, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS_BYTES));
-    CUDA_OK(cudaFuncSetAttribute(k_batch_step<float, BLK, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS_BYTES));
-    attr = true;
-  }
+  // before any capture of the packed steps
+  if (!(precision == LBM39_MIXED
+            ? allow_shared<k_batch_step<float, Launch<float>::BLK, false>>(Launch<float>::WSB)
+            : allow_shared<k_batch_step<double, Launch<double>::BLK, true>>(Launch<double>::WSB) &&
+                  allow_shared<k_batch_step<double, Launch<double>::BLK, false>>(
+                      Launch<double>::WSB)))
+    return LBM39_ERR_CUDA;
   lbm39_batch* B = new (std::nothrow) lbm39_batch;
   if (!B) return LBM39_ERR_ARG;
   const BatchLayout lay = batch_layout(max_lattices, max_cells);
@@ -876,7 +889,7 @@ int lbm39_batch_set(lbm39_batch* B, lbm39_lattice* const* lattices, const int64_
     B->tend.push_back(t_end[j]);
     // the nine-constraint (z-mirror) tiles first: they take their own instantiation
     std::vector<Tile>& dst = (!L->mixed && L->desc.d2) ? B->hT : full;
-    for (long long c = 0; c < L->N; c += BLK) dst.push_back(Tile{j, 0, c});
+    for (long long c = 0; c < L->N; c += tile_cells(B->precision)) dst.push_back(Tile{j, 0, c});
     if (L->fills)
       for (long long c = 0; c < L->N; c += 256) B->hF.push_back(Tile{j, 0, c});
   }

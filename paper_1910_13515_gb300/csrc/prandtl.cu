@@ -13,19 +13,19 @@
 namespace lbm39 {
 
 namespace {
-constexpr int BLK = 64;  // the step kernel's block (the workspace is laid out per block)
-constexpr size_t WS_BYTES = (size_t)BLK * WS_DOUBLES * sizeof(double);
+template <class P>
+void launch(const Desc& d, bool odd, cudaStream_t stream) {
+  constexpr bool FIXED = in_fixed_point<P, 0>;
+  constexpr int BLK = solve_blk(FIXED);
+  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
+  if (odd) launch_ws<k_step<true, P, BLK, false, true>>(grid, BLK, ws_bytes(FIXED), stream, d);
+  else launch_ws<k_step<false, P, BLK, false, true>>(grid, BLK, ws_bytes(FIXED), stream, d);
+}
 }  // namespace
 
 bool launch_step_prandtl(const Desc& d, bool odd, bool mixed, cudaStream_t stream) {
-  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
-  if (mixed) {
-    if (odd) k_step<true, float, BLK, false, true><<<grid, BLK, WS_BYTES, stream>>>(d);
-    else k_step<false, float, BLK, false, true><<<grid, BLK, WS_BYTES, stream>>>(d);
-  } else {
-    if (odd) k_step<true, double, BLK, false, true><<<grid, BLK, WS_BYTES, stream>>>(d);
-    else k_step<false, double, BLK, false, true><<<grid, BLK, WS_BYTES, stream>>>(d);
-  }
+  if (mixed) launch<float>(d, odd, stream);
+  else launch<double>(d, odd, stream);
   return cudaGetLastError() == cudaSuccess;
 }
 

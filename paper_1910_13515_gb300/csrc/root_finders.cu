@@ -13,26 +13,25 @@
 namespace lbm39 {
 
 namespace {
-constexpr int BLK = 64;  // the step kernel's block (the workspace is laid out per block)
-constexpr size_t WS_BYTES = (size_t)BLK * WS_DOUBLES * sizeof(double);
-
 template <int SOLVER>
-void launch(const Desc& d, bool odd, cudaStream_t stream, unsigned grid) {
+void launch(const Desc& d, bool odd, cudaStream_t stream) {
+  constexpr bool FIXED = in_fixed_point<double, SOLVER>;
+  constexpr int BLK = solve_blk(FIXED);
+  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
   if (d.d2) {
-    if (odd) k_step<true, double, BLK, true, false, SOLVER><<<grid, BLK, WS_BYTES, stream>>>(d);
-    else k_step<false, double, BLK, true, false, SOLVER><<<grid, BLK, WS_BYTES, stream>>>(d);
+    if (odd) launch_ws<k_step<true, double, BLK, true, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
+    else launch_ws<k_step<false, double, BLK, true, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
   } else {
-    if (odd) k_step<true, double, BLK, false, false, SOLVER><<<grid, BLK, WS_BYTES, stream>>>(d);
-    else k_step<false, double, BLK, false, false, SOLVER><<<grid, BLK, WS_BYTES, stream>>>(d);
+    if (odd) launch_ws<k_step<true, double, BLK, false, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
+    else launch_ws<k_step<false, double, BLK, false, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
   }
 }
 }  // namespace
 
 bool launch_step_root_finder(const Desc& d, bool odd, int solver, cudaStream_t stream) {
-  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
-  if (solver == 1) launch<1>(d, odd, stream, grid);
-  else if (solver == 2) launch<2>(d, odd, stream, grid);
-  else if (solver == 3) launch<3>(d, odd, stream, grid);
+  if (solver == 1) launch<1>(d, odd, stream);
+  else if (solver == 2) launch<2>(d, odd, stream);
+  else if (solver == 3) launch<3>(d, odd, stream);
   else return false;
   return cudaGetLastError() == cudaSuccess;
 }
