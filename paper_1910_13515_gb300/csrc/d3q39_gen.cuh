@@ -1588,6 +1588,161 @@ __device__ __forceinline__ void jvec_fx(const int (&d)[13], const V& p, unsigned
   s[10] += 27ull * w13_0_1;
 }
 
+// sum_i v(i) [1, xi_i, |xi_i|^2] in 64-bit integers.
+template <class V>
+__device__ __forceinline__ void macro_fx(const V& v, unsigned long long (&s)[5]) {
+  const unsigned long long v0 = v(Idx<0>{});
+  s[0] = v0;
+  const unsigned long long v5 = v(Idx<5>{});
+  const unsigned long long v6 = v(Idx<6>{});
+  const unsigned long long w1_0_0 = v5 + v6;
+  const unsigned long long w1_0_1 = v5 - v6;
+  s[0] += w1_0_0;
+  s[4] = w1_0_0;
+  s[3] = w1_0_1;
+  const unsigned long long v19 = v(Idx<19>{});
+  const unsigned long long v20 = v(Idx<20>{});
+  const unsigned long long w2_0_0 = v19 + v20;
+  const unsigned long long w2_0_1 = v19 - v20;
+  s[0] += w2_0_0;
+  s[4] += 4ull * w2_0_0;
+  s[3] += 2ull * w2_0_1;
+  const unsigned long long v37 = v(Idx<37>{});
+  const unsigned long long v38 = v(Idx<38>{});
+  const unsigned long long w3_0_0 = v37 + v38;
+  const unsigned long long w3_0_1 = v37 - v38;
+  s[0] += w3_0_0;
+  s[4] += 9ull * w3_0_0;
+  s[3] += 3ull * w3_0_1;
+  const unsigned long long v3 = v(Idx<3>{});
+  const unsigned long long v4 = v(Idx<4>{});
+  const unsigned long long w4_0_0 = v3 + v4;
+  const unsigned long long w4_0_1 = v3 - v4;
+  s[0] += w4_0_0;
+  s[4] += w4_0_0;
+  s[2] = w4_0_1;
+  const unsigned long long v17 = v(Idx<17>{});
+  const unsigned long long v18 = v(Idx<18>{});
+  const unsigned long long w5_0_0 = v17 + v18;
+  const unsigned long long w5_0_1 = v17 - v18;
+  s[0] += w5_0_0;
+  s[4] += 4ull * w5_0_0;
+  s[2] += 2ull * w5_0_1;
+  const unsigned long long v29 = v(Idx<29>{});
+  const unsigned long long v30 = v(Idx<30>{});
+  const unsigned long long v31 = v(Idx<31>{});
+  const unsigned long long v32 = v(Idx<32>{});
+  const unsigned long long w6_0_0 = v31 + v30;
+  const unsigned long long w6_0_1 = v31 - v30;
+  const unsigned long long w6_0_2 = v29 + v32;
+  const unsigned long long w6_0_3 = v29 - v32;
+  const unsigned long long w6_1_0 = w6_0_2 + w6_0_0;
+  const unsigned long long w6_1_1 = w6_0_2 - w6_0_0;
+  const unsigned long long w6_1_2 = w6_0_3 + w6_0_1;
+  const unsigned long long w6_1_3 = w6_0_3 - w6_0_1;
+  s[0] += w6_1_0;
+  s[4] += 8ull * w6_1_0;
+  s[3] += 2ull * w6_1_1;
+  s[2] += 2ull * w6_1_2;
+  const unsigned long long v35 = v(Idx<35>{});
+  const unsigned long long v36 = v(Idx<36>{});
+  const unsigned long long w7_0_0 = v35 + v36;
+  const unsigned long long w7_0_1 = v35 - v36;
+  s[0] += w7_0_0;
+  s[4] += 9ull * w7_0_0;
+  s[2] += 3ull * w7_0_1;
+  const unsigned long long v1 = v(Idx<1>{});
+  const unsigned long long v2 = v(Idx<2>{});
+  const unsigned long long w8_0_0 = v1 + v2;
+  const unsigned long long w8_0_1 = v1 - v2;
+  s[0] += w8_0_0;
+  s[4] += w8_0_0;
+  s[1] = w8_0_1;
+  const unsigned long long v7 = v(Idx<7>{});
+  const unsigned long long v8 = v(Idx<8>{});
+  const unsigned long long v9 = v(Idx<9>{});
+  const unsigned long long v10 = v(Idx<10>{});
+  const unsigned long long v11 = v(Idx<11>{});
+  const unsigned long long v12 = v(Idx<12>{});
+  const unsigned long long v13 = v(Idx<13>{});
+  const unsigned long long v14 = v(Idx<14>{});
+  const unsigned long long w9_0_0 = v14 + v8;
+  const unsigned long long w9_0_1 = v14 - v8;
+  const unsigned long long w9_0_2 = v11 + v10;
+  const unsigned long long w9_0_3 = v11 - v10;
+  const unsigned long long w9_0_4 = v9 + v12;
+  const unsigned long long w9_0_5 = v9 - v12;
+  const unsigned long long w9_0_6 = v7 + v13;
+  const unsigned long long w9_0_7 = v7 - v13;
+  const unsigned long long w9_1_0 = w9_0_4 + w9_0_0;
+  const unsigned long long w9_1_1 = w9_0_4 - w9_0_0;
+  const unsigned long long w9_1_2 = w9_0_6 + w9_0_2;
+  const unsigned long long w9_1_3 = w9_0_6 - w9_0_2;
+  const unsigned long long w9_1_4 = w9_0_5 + w9_0_1;
+  const unsigned long long w9_1_5 = w9_0_5 - w9_0_1;
+  const unsigned long long w9_1_6 = w9_0_7 + w9_0_3;
+  const unsigned long long w9_1_7 = w9_0_7 - w9_0_3;
+  const unsigned long long w9_2_0 = w9_1_2 + w9_1_0;
+  const unsigned long long w9_2_1 = w9_1_2 - w9_1_0;
+  const unsigned long long w9_2_2 = w9_1_3 + w9_1_1;
+  const unsigned long long w9_2_3 = w9_1_3 - w9_1_1;
+  const unsigned long long w9_2_4 = w9_1_6 + w9_1_4;
+  const unsigned long long w9_2_5 = w9_1_6 - w9_1_4;
+  const unsigned long long w9_2_6 = w9_1_7 + w9_1_5;
+  const unsigned long long w9_2_7 = w9_1_7 - w9_1_5;
+  s[0] += w9_2_0;
+  s[4] += 3ull * w9_2_0;
+  s[3] += w9_2_1;
+  s[2] += w9_2_2;
+  s[1] += w9_2_4;
+  const unsigned long long v15 = v(Idx<15>{});
+  const unsigned long long v16 = v(Idx<16>{});
+  const unsigned long long w10_0_0 = v15 + v16;
+  const unsigned long long w10_0_1 = v15 - v16;
+  s[0] += w10_0_0;
+  s[4] += 4ull * w10_0_0;
+  s[1] += 2ull * w10_0_1;
+  const unsigned long long v25 = v(Idx<25>{});
+  const unsigned long long v26 = v(Idx<26>{});
+  const unsigned long long v27 = v(Idx<27>{});
+  const unsigned long long v28 = v(Idx<28>{});
+  const unsigned long long w11_0_0 = v27 + v26;
+  const unsigned long long w11_0_1 = v27 - v26;
+  const unsigned long long w11_0_2 = v25 + v28;
+  const unsigned long long w11_0_3 = v25 - v28;
+  const unsigned long long w11_1_0 = w11_0_2 + w11_0_0;
+  const unsigned long long w11_1_1 = w11_0_2 - w11_0_0;
+  const unsigned long long w11_1_2 = w11_0_3 + w11_0_1;
+  const unsigned long long w11_1_3 = w11_0_3 - w11_0_1;
+  s[0] += w11_1_0;
+  s[4] += 8ull * w11_1_0;
+  s[3] += 2ull * w11_1_1;
+  s[1] += 2ull * w11_1_2;
+  const unsigned long long v21 = v(Idx<21>{});
+  const unsigned long long v22 = v(Idx<22>{});
+  const unsigned long long v23 = v(Idx<23>{});
+  const unsigned long long v24 = v(Idx<24>{});
+  const unsigned long long w12_0_0 = v23 + v22;
+  const unsigned long long w12_0_1 = v23 - v22;
+  const unsigned long long w12_0_2 = v21 + v24;
+  const unsigned long long w12_0_3 = v21 - v24;
+  const unsigned long long w12_1_0 = w12_0_2 + w12_0_0;
+  const unsigned long long w12_1_1 = w12_0_2 - w12_0_0;
+  const unsigned long long w12_1_2 = w12_0_3 + w12_0_1;
+  const unsigned long long w12_1_3 = w12_0_3 - w12_0_1;
+  s[0] += w12_1_0;
+  s[4] += 8ull * w12_1_0;
+  s[2] += 2ull * w12_1_1;
+  s[1] += 2ull * w12_1_2;
+  const unsigned long long v33 = v(Idx<33>{});
+  const unsigned long long v34 = v(Idx<34>{});
+  const unsigned long long w13_0_0 = v33 + v34;
+  const unsigned long long w13_0_1 = v33 - v34;
+  s[0] += w13_0_0;
+  s[4] += 9ull * w13_0_0;
+  s[1] += 3ull * w13_0_1;
+}
+
 // s_k = sum_i v(i) phi_k(xi_i) in 64-bit integers (the nine z-even k, values mirror-symmetric in z).
 template <class V>
 __device__ __forceinline__ void sums_fx2d(const V& v, unsigned long long (&s)[9]) {
@@ -1619,9 +1774,9 @@ __device__ __forceinline__ void sums_fx2d(const V& v, unsigned long long (&s)[9]
   s[2] += 2ull * w5_0_1;
   s[8] += 8ull * w5_0_1;
   const unsigned long long v29 = v(Idx<29>{});
-  const unsigned long long v32 = v(Idx<32>{});
-  const unsigned long long w6_0_0 = v29 + v32;
-  const unsigned long long w6_0_1 = v29 - v32;
+  const unsigned long long v30 = v(Idx<30>{});
+  const unsigned long long w6_0_0 = v29 + v30;
+  const unsigned long long w6_0_1 = v29 - v30;
   s[0] += 2ull * w6_0_0;
   s[4] += 8ull * w6_0_0;
   s[5] += 8ull * w6_0_0;
@@ -1644,13 +1799,13 @@ __device__ __forceinline__ void sums_fx2d(const V& v, unsigned long long (&s)[9]
   s[1] = w8_0_1;
   s[7] = w8_0_1;
   const unsigned long long v7 = v(Idx<7>{});
-  const unsigned long long v10 = v(Idx<10>{});
+  const unsigned long long v8 = v(Idx<8>{});
   const unsigned long long v11 = v(Idx<11>{});
-  const unsigned long long v13 = v(Idx<13>{});
-  const unsigned long long w9_0_0 = v11 + v10;
-  const unsigned long long w9_0_1 = v11 - v10;
-  const unsigned long long w9_0_2 = v7 + v13;
-  const unsigned long long w9_0_3 = v7 - v13;
+  const unsigned long long v12 = v(Idx<12>{});
+  const unsigned long long w9_0_0 = v11 + v8;
+  const unsigned long long w9_0_1 = v11 - v8;
+  const unsigned long long w9_0_2 = v7 + v12;
+  const unsigned long long w9_0_3 = v7 - v12;
   const unsigned long long w9_1_0 = w9_0_2 + w9_0_0;
   const unsigned long long w9_1_1 = w9_0_2 - w9_0_0;
   const unsigned long long w9_1_2 = w9_0_3 + w9_0_1;
@@ -1673,9 +1828,9 @@ __device__ __forceinline__ void sums_fx2d(const V& v, unsigned long long (&s)[9]
   s[1] += 2ull * w10_0_1;
   s[7] += 8ull * w10_0_1;
   const unsigned long long v25 = v(Idx<25>{});
-  const unsigned long long v28 = v(Idx<28>{});
-  const unsigned long long w11_0_0 = v25 + v28;
-  const unsigned long long w11_0_1 = v25 - v28;
+  const unsigned long long v26 = v(Idx<26>{});
+  const unsigned long long w11_0_0 = v25 + v26;
+  const unsigned long long w11_0_1 = v25 - v26;
   s[0] += 2ull * w11_0_0;
   s[3] += 8ull * w11_0_0;
   s[5] += 8ull * w11_0_0;
@@ -1758,9 +1913,9 @@ __device__ __forceinline__ void jvec_fx2d(const int (&d)[9], const V& p, unsigne
   const int y6_0_0 = c6_0 + c6_y;
   const int y6_0_1 = c6_0 - c6_y;
   const unsigned long long p29 = p(Idx<29>{}, y6_0_0);
-  const unsigned long long p32 = p(Idx<32>{}, y6_0_1);
-  const unsigned long long w6_0_0 = p29 + p32;
-  const unsigned long long w6_0_1 = p29 - p32;
+  const unsigned long long p30 = p(Idx<30>{}, y6_0_1);
+  const unsigned long long w6_0_0 = p29 + p30;
+  const unsigned long long w6_0_1 = p29 - p30;
   s[0] += 2ull * w6_0_0;
   s[4] += 8ull * w6_0_0;
   s[5] += 8ull * w6_0_0;
@@ -1803,13 +1958,13 @@ __device__ __forceinline__ void jvec_fx2d(const int (&d)[9], const V& p, unsigne
   const int y9_1_2 = y9_0_0 + y9_0_2;
   const int y9_1_3 = y9_0_0 - y9_0_2;
   const unsigned long long p7 = p(Idx<7>{}, y9_1_2);
-  const unsigned long long p10 = p(Idx<10>{}, y9_1_1);
+  const unsigned long long p8 = p(Idx<8>{}, y9_1_1);
   const unsigned long long p11 = p(Idx<11>{}, y9_1_3);
-  const unsigned long long p13 = p(Idx<13>{}, y9_1_0);
-  const unsigned long long w9_0_0 = p11 + p10;
-  const unsigned long long w9_0_1 = p11 - p10;
-  const unsigned long long w9_0_2 = p7 + p13;
-  const unsigned long long w9_0_3 = p7 - p13;
+  const unsigned long long p12 = p(Idx<12>{}, y9_1_0);
+  const unsigned long long w9_0_0 = p11 + p8;
+  const unsigned long long w9_0_1 = p11 - p8;
+  const unsigned long long w9_0_2 = p7 + p12;
+  const unsigned long long w9_0_3 = p7 - p12;
   const unsigned long long w9_1_0 = w9_0_2 + w9_0_0;
   const unsigned long long w9_1_1 = w9_0_2 - w9_0_0;
   const unsigned long long w9_1_2 = w9_0_3 + w9_0_1;
@@ -1840,9 +1995,9 @@ __device__ __forceinline__ void jvec_fx2d(const int (&d)[9], const V& p, unsigne
   const int y11_0_0 = c11_0 + c11_x;
   const int y11_0_1 = c11_0 - c11_x;
   const unsigned long long p25 = p(Idx<25>{}, y11_0_0);
-  const unsigned long long p28 = p(Idx<28>{}, y11_0_1);
-  const unsigned long long w11_0_0 = p25 + p28;
-  const unsigned long long w11_0_1 = p25 - p28;
+  const unsigned long long p26 = p(Idx<26>{}, y11_0_1);
+  const unsigned long long w11_0_0 = p25 + p26;
+  const unsigned long long w11_0_1 = p25 - p26;
   s[0] += 2ull * w11_0_0;
   s[3] += 8ull * w11_0_0;
   s[5] += 8ull * w11_0_0;
@@ -1892,6 +2047,110 @@ __device__ __forceinline__ void jvec_fx2d(const int (&d)[9], const V& p, unsigne
   s[3] += 9ull * w13_0_0;
   s[1] += 3ull * w13_0_1;
   s[7] += 27ull * w13_0_1;
+}
+
+// sum_i v(i) [1, xi_i, |xi_i|^2] in 64-bit integers (values mirror-symmetric in z: no xi_z).
+template <class V>
+__device__ __forceinline__ void macro_fx2d(const V& v, unsigned long long (&s)[4]) {
+  const unsigned long long v0 = v(Idx<0>{});
+  s[0] = v0;
+  const unsigned long long v5 = v(Idx<5>{});
+  s[0] += 2ull * v5;
+  s[3] = 2ull * v5;
+  const unsigned long long v19 = v(Idx<19>{});
+  s[0] += 2ull * v19;
+  s[3] += 8ull * v19;
+  const unsigned long long v37 = v(Idx<37>{});
+  s[0] += 2ull * v37;
+  s[3] += 18ull * v37;
+  const unsigned long long v3 = v(Idx<3>{});
+  const unsigned long long v4 = v(Idx<4>{});
+  const unsigned long long w4_0_0 = v3 + v4;
+  const unsigned long long w4_0_1 = v3 - v4;
+  s[0] += w4_0_0;
+  s[3] += w4_0_0;
+  s[2] = w4_0_1;
+  const unsigned long long v17 = v(Idx<17>{});
+  const unsigned long long v18 = v(Idx<18>{});
+  const unsigned long long w5_0_0 = v17 + v18;
+  const unsigned long long w5_0_1 = v17 - v18;
+  s[0] += w5_0_0;
+  s[3] += 4ull * w5_0_0;
+  s[2] += 2ull * w5_0_1;
+  const unsigned long long v29 = v(Idx<29>{});
+  const unsigned long long v30 = v(Idx<30>{});
+  const unsigned long long w6_0_0 = v29 + v30;
+  const unsigned long long w6_0_1 = v29 - v30;
+  s[0] += 2ull * w6_0_0;
+  s[3] += 16ull * w6_0_0;
+  s[2] += 4ull * w6_0_1;
+  const unsigned long long v35 = v(Idx<35>{});
+  const unsigned long long v36 = v(Idx<36>{});
+  const unsigned long long w7_0_0 = v35 + v36;
+  const unsigned long long w7_0_1 = v35 - v36;
+  s[0] += w7_0_0;
+  s[3] += 9ull * w7_0_0;
+  s[2] += 3ull * w7_0_1;
+  const unsigned long long v1 = v(Idx<1>{});
+  const unsigned long long v2 = v(Idx<2>{});
+  const unsigned long long w8_0_0 = v1 + v2;
+  const unsigned long long w8_0_1 = v1 - v2;
+  s[0] += w8_0_0;
+  s[3] += w8_0_0;
+  s[1] = w8_0_1;
+  const unsigned long long v7 = v(Idx<7>{});
+  const unsigned long long v8 = v(Idx<8>{});
+  const unsigned long long v11 = v(Idx<11>{});
+  const unsigned long long v12 = v(Idx<12>{});
+  const unsigned long long w9_0_0 = v11 + v8;
+  const unsigned long long w9_0_1 = v11 - v8;
+  const unsigned long long w9_0_2 = v7 + v12;
+  const unsigned long long w9_0_3 = v7 - v12;
+  const unsigned long long w9_1_0 = w9_0_2 + w9_0_0;
+  const unsigned long long w9_1_1 = w9_0_2 - w9_0_0;
+  const unsigned long long w9_1_2 = w9_0_3 + w9_0_1;
+  const unsigned long long w9_1_3 = w9_0_3 - w9_0_1;
+  s[0] += 2ull * w9_1_0;
+  s[3] += 6ull * w9_1_0;
+  s[2] += 2ull * w9_1_1;
+  s[1] += 2ull * w9_1_2;
+  const unsigned long long v15 = v(Idx<15>{});
+  const unsigned long long v16 = v(Idx<16>{});
+  const unsigned long long w10_0_0 = v15 + v16;
+  const unsigned long long w10_0_1 = v15 - v16;
+  s[0] += w10_0_0;
+  s[3] += 4ull * w10_0_0;
+  s[1] += 2ull * w10_0_1;
+  const unsigned long long v25 = v(Idx<25>{});
+  const unsigned long long v26 = v(Idx<26>{});
+  const unsigned long long w11_0_0 = v25 + v26;
+  const unsigned long long w11_0_1 = v25 - v26;
+  s[0] += 2ull * w11_0_0;
+  s[3] += 16ull * w11_0_0;
+  s[1] += 4ull * w11_0_1;
+  const unsigned long long v21 = v(Idx<21>{});
+  const unsigned long long v22 = v(Idx<22>{});
+  const unsigned long long v23 = v(Idx<23>{});
+  const unsigned long long v24 = v(Idx<24>{});
+  const unsigned long long w12_0_0 = v23 + v22;
+  const unsigned long long w12_0_1 = v23 - v22;
+  const unsigned long long w12_0_2 = v21 + v24;
+  const unsigned long long w12_0_3 = v21 - v24;
+  const unsigned long long w12_1_0 = w12_0_2 + w12_0_0;
+  const unsigned long long w12_1_1 = w12_0_2 - w12_0_0;
+  const unsigned long long w12_1_2 = w12_0_3 + w12_0_1;
+  const unsigned long long w12_1_3 = w12_0_3 - w12_0_1;
+  s[0] += w12_1_0;
+  s[3] += 8ull * w12_1_0;
+  s[2] += 2ull * w12_1_1;
+  s[1] += 2ull * w12_1_2;
+  const unsigned long long v33 = v(Idx<33>{});
+  const unsigned long long v34 = v(Idx<34>{});
+  const unsigned long long w13_0_0 = v33 + v34;
+  const unsigned long long w13_0_1 = v33 - v34;
+  s[0] += w13_0_0;
+  s[3] += 9ull * w13_0_0;
+  s[1] += 3ull * w13_0_1;
 }
 
 // 2^(j/1024) in units of 2^-55, j = 0..1023, each the integer nearest the exact value.

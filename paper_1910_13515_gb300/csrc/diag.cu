@@ -31,14 +31,13 @@ __device__ __forceinline__ void gather_f(const Desc& d, long long cell, double (
   }
 }
 
-template <class P>
-__device__ __forceinline__ Macro moments_at(const Desc& d, long long cell, bool odd) {
+// The step's own macroscopic variables (the same arithmetic, so the same updates).
+template <bool ODD, class P, bool D2, bool FIXED>
+__device__ __forceinline__ Macro moments_of(const Desc& d, long long cell) {
   Nbr nb;
-  if (odd) {
-    nb = Nbr(d, coord_of(d, cell));
-    return gather_moments<true, P>(d, cell, nb);
-  }
-  return gather_moments<false, P>(d, cell, nb);
+  if constexpr (ODD) nb = Nbr(d, coord_of(d, cell));
+  if constexpr (FIXED) return step_moments<ODD, D2>(d, cell, nb);
+  else return gather_moments<ODD, P>(d, cell, nb);
 }
 
 // eps: FP64 (1/Q) sum_i |f_i - f_i^eq| / f_i^eq of the state against the
@@ -61,13 +60,15 @@ __global__ void __launch_bounds__(solve_blk(in_fixed_point<P, SOLVER>))
   }
   WS<BLK> w{smem + threadIdx.x};
   WS<BLK> F = w.at(WS_E), lam = w.at(WS_LAM), m = w.at(WS_M);
-  const Macro M = moments_at<P>(d, cell, odd != 0);
+  const Macro M = odd ? moments_of<true, P, D2, FIXED>(d, cell)
+                      : moments_of<false, P, D2, FIXED>(d, cell);
   targets<BLK>(M.ux, M.uy, M.uz, M.T, m);
   load_solver_state<BLK>(d, cell, w);
   const bool marked = is_fallback_embedding<BLK>(lam);
   const int maxit = !marked ? d.ph.maxit : retry_budget(d.t, d.ph.maxit);
   int n32;
-  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32);
+  bool moved;
+  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32, moved);
   if (nr.failed) {
     targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // the solve may have overwritten them
     fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);

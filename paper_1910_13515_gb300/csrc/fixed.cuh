@@ -109,12 +109,13 @@ __device__ __forceinline__ double exp2_fixed(s64 X, const u64* __restrict__ tab)
   return __hiloint2double((int)((unsigned)(m >> 32) + e), (int)(unsigned)m);
 }
 
-// A double in (0, 0.75) as an integer in units 2^-58, rounded down.
-__device__ __forceinline__ u64 unit58(double F) {
+// F 2^(1023 - top) as an integer in units 2^-58, rounded down, for F > 0 with F 2^(1023 - top)
+// below 2.
+__device__ __forceinline__ u64 unit58(double F, int top = 1023) {
   const unsigned hi = (unsigned)__double2hiint(F), lo = (unsigned)__double2loint(F);
   const unsigned mh = (hi & 0xfffffu) | 0x100000u;
   const u64 m = ((u64)__funnelshift_l(lo, mh, 6) << 32) | (lo << 6);
-  const unsigned s = min(1023u - (hi >> 20), 63u);
+  const unsigned s = min((unsigned)top - (hi >> 20), 63u);
   return m >> s;
 }
 

@@ -19,6 +19,7 @@ Emitted:
   f_moments(f, ...)           rho, j, sum f|xi|^2;  g_sum(g): sum g
   exp2_table                  2^(j/256), j = 0..255, correctly rounded (decimal arithmetic)
   sums_fx, sums_fx2d          sum_i v(i) phi_k(xi_i) in 64-bit integers, orbit by orbit
+  macro_fx, macro_fx2d        sum_i v(i) [1, xi_i, |xi_i|^2] likewise
   jvec_fx, jvec_fx2d          sum_i p(i, y_i) phi_k(xi_i) with y_i = sum_k d_k phi_k(xi_i)
   exp2_fixed                  2^(j/1024) 2^55, j = 0..1023, nearest integers
   exp constants               ln2/256 split in a 32-bit head and a tail
@@ -427,13 +428,16 @@ def exp_constants():
 # not matter, and the z-mirror form (basis functions even in xi_z, values equal under the mirror)
 # reads one velocity of each mirror pair and counts it twice with the same result.
 
-def _orbit_terms(ks):
-    """Per orbit: {sign subset T: [(result index, integer factor)]} of the basis functions ks."""
+# rho, j, sum f |xi|^2
+MACRO_BASIS = [((0, 0, 0), 0), ((1, 0, 0), 0), ((0, 1, 0), 0), ((0, 0, 1), 0), ((0, 0, 0), 1)]
+
+
+def _orbit_terms(basis):
+    """Per orbit: {sign subset T: [(result index, integer factor)]} of the basis functions."""
     out = []
     for key, axes, members in ORBITS:
         use = {}
-        for pos, k in enumerate(ks):
-            p, m = GBASIS[k]
+        for pos, (p, m) in enumerate(basis):
             if any(p[a] != 0 and key[a] == 0 for a in range(3)):
                 continue
             mag = sum(c * c for c in key) ** m
@@ -445,13 +449,20 @@ def _orbit_terms(ks):
     return out
 
 
-def gen_int_sums(zsym=False, jvec=False):
+def gen_int_sums(zsym=False, jvec=False, macro=False):
     em = Emitter()
     ks = ZEVEN if zsym else list(range(NM))
-    n = len(ks)
-    name = ("jvec_fx" if jvec else "sums_fx") + ("2d" if zsym else "")
-    em(f"// s_k = sum_i {'p(i, y_i)' if jvec else 'v(i)'} phi_k(xi_i) in 64-bit integers"
-       + (" (the nine z-even k, values mirror-symmetric in z)." if zsym else "."))
+    basis = [GBASIS[k] for k in ks]
+    if macro:
+        basis = [b for b in MACRO_BASIS if not (zsym and b[0][2] % 2)]
+    n = len(basis)
+    name = ("macro_fx" if macro else "jvec_fx" if jvec else "sums_fx") + ("2d" if zsym else "")
+    if macro:
+        em("// sum_i v(i) [1, xi_i, |xi_i|^2] in 64-bit integers"
+           + (" (values mirror-symmetric in z: no xi_z)." if zsym else "."))
+    else:
+        em(f"// s_k = sum_i {'p(i, y_i)' if jvec else 'v(i)'} phi_k(xi_i) in 64-bit integers"
+           + (" (the nine z-even k, values mirror-symmetric in z)." if zsym else "."))
     em("template <class V>")
     if jvec:
         em(f"__device__ __forceinline__ void {name}(const int (&d)[{n}], const V& p, "
@@ -459,15 +470,15 @@ def gen_int_sums(zsym=False, jvec=False):
     else:
         em(f"__device__ __forceinline__ void {name}(const V& v, unsigned long long (&s)[{n}]) {{")
     first = [True] * n
-    for o, ((key, axes, members), use) in enumerate(zip(ORBITS, _orbit_terms(ks))):
+    for o, ((key, axes, members), use) in enumerate(zip(ORBITS, _orbit_terms(basis))):
         # a z-mirror pair enters once: fold over the other axes only
         ax = [a for a in axes if not (zsym and a == 2)]
         double = 2 if zsym and 2 in axes else 1
         mem = {}
         for sg, i in members.items():
             sd = dict(zip(axes, sg))
-            if zsym and 2 in axes and sd[2] < 0:
-                continue
+            if zsym and VEL.index((VEL[i][0], VEL[i][1], -VEL[i][2])) < i:
+                continue  # the first of a mirror pair stands for both
             mem[tuple(sd[a] for a in ax)] = i
         cur = {}
         if jvec:  # y of the orbit's members: coefficients of the sign subsets, then butterflies
@@ -537,7 +548,7 @@ def gen_int_sums(zsym=False, jvec=False):
     return em.lines
 
 
-def selfcheck_int(lines, zsym, jvec):
+def selfcheck_int(lines, zsym, jvec, macro=False):
     """The emitted integer sums against direct sums over the 39 velocities."""
     import random
     import re
@@ -556,6 +567,12 @@ def selfcheck_int(lines, zsym, jvec):
         t = re.sub(r"^const (int|unsigned long long) ", "", t).rstrip(";")
         # `p` and `v` are both functions and prefixes of names: names carry a digit
         exec(t, env)
+    if macro:
+        for pos, (pw, m) in enumerate(b for b in MACRO_BASIS if not (zsym and b[0][2] % 2)):
+            ref = sum(F[i] * sum(c * c for c in v) ** m * v[0] ** pw[0] * v[1] ** pw[1]
+                      * v[2] ** pw[2] for i, v in enumerate(VEL))
+            assert env["s"][pos] == ref, (zsym, pos)
+        return
     for pos, k in enumerate(ks):
         ref = sum((F[i] * y[i] if jvec else F[i]) * phi(k, VEL[i]) for i in range(Q))
         assert env["s"][pos] == ref, (zsym, jvec, k)
@@ -725,6 +742,9 @@ def generate():
             body = gen_int_sums(zsym, jvec)
             selfcheck_int(body, zsym, jvec)
             int_lines += [""] + body
+        body = gen_int_sums(zsym, macro=True)
+        selfcheck_int(body, zsym, False, macro=True)
+        int_lines += [""] + body
     lines += int_lines
     lines.append("")
     lines.append("// 2^(j/1024) in units of 2^-55, j = 0..1023, each the integer nearest the exact value.")

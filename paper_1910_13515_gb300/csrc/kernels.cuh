@@ -68,11 +68,12 @@ __device__ __forceinline__ Coord coord_of(const Desc& d, long long cell) {
   return Coord{c - yz * d.nx, yz % d.ny, yz / d.ny};
 }
 
-// a mod n for a in [-3, n + 2]: one conditional correction when n >= 3.
+// a mod n for a in [-3, n + 2]: one conditional correction when n >= 3, the last bit or 0 below.
+// (Written with the remainder operator, the 21 wraps of a neighbour table were 2000 instructions
+// in each of the odd pass's two tables, a third of the kernel.)
 __device__ __forceinline__ int wrap(int a, int n) {
-  if (n >= 3) return a < 0 ? a + n : (a >= n ? a - n : a);
-  const int r = a % n;
-  return r < 0 ? r + n : r;
+  const int add = n >= 3 ? n : 0, mask = n >= 3 ? -1 : n - 1;
+  return (a + (a < 0 ? add : 0) - (a >= n ? add : 0)) & mask;
 }
 
 // Index of the cell at x + (dx, dy, dz) with periodic wrap of every axis
@@ -107,22 +108,36 @@ __device__ __forceinline__ Nbr fresh_nbr(const Desc& d, Coord c) {
   return nb;
 }
 
+// Element at an index of a plane.  The plane's address is the same for all threads, and the byte
+// offset in it fits in 32 bits (a plane of 2^32 bytes is one of 2^29 doubles, and the 130 planes of
+// such a lattice are twice the memory of a GB300): one instruction with a uniform base and a 32-bit
+// offset, where 64-bit addresses took ten for each of a cell's 300 accesses.
+template <class P>
+__device__ __forceinline__ P& at(P* plane, int index) {
+  return *reinterpret_cast<P*>(reinterpret_cast<char*>(const_cast<std::remove_const_t<P>*>(plane)) +
+                               (unsigned)index * (unsigned)sizeof(P));
+}
+
 // Pre-collision populations of one distribution (base 0: f, Q: g) of fluid
 // cell `cell` at the lattice's current time: own slots at even time, the odd
 // gather from (x - xi_i, slot opp i) at odd time.  Where x - xi_i is solid,
 // that slot holds the bounced population (bounce_even_cell), so the gather
 // has no per-direction branch.
-template <bool ODD, class P>
+// D2 (the z-mirror-symmetric lattices): one of each mirror pair is read; they
+// are equal bit for bit.
+template <bool ODD, class P, bool D2 = false>
 __device__ __forceinline__ void gather(const Desc& d, long long cell, const Nbr& nb, int base,
                                        P (&h)[Q]) {
   const P* __restrict__ pop = static_cast<const P*>(d.pop);
   static_for<0, Q>([&](auto I) {
     constexpr int i = decltype(I)::value;
-    if constexpr (!ODD) {
-      h[i] = pop[(long long)(base + i) * d.Np + cell];
+    if constexpr (D2 && zmirror(i) < i) {
+      h[i] = h[zmirror(i)];
+    } else if constexpr (!ODD) {
+      h[i] = at(pop + (long long)(base + i) * d.Np, (int)cell);
     } else {
       constexpr int cx = CX[i], cy = CY[i], cz = CZ[i];
-      h[i] = pop[(long long)(base + opp(i)) * d.Np + nb.at(-cx, -cy, -cz)];
+      h[i] = at(pop + (long long)(base + opp(i)) * d.Np, nb.at(-cx, -cy, -cz));
     }
   });
 }
@@ -135,11 +150,20 @@ __device__ __forceinline__ void push(const Desc& d, long long cell, const Nbr& n
                                      P v) {
   P* __restrict__ pop = static_cast<P*>(d.pop);
   if constexpr (!ODD) {
-    pop[(long long)(base + opp(i)) * d.Np + cell] = v;
+    at(pop + (long long)(base + opp(i)) * d.Np, (int)cell) = v;
   } else {
     constexpr int cx = CX[i], cy = CY[i], cz = CZ[i];
-    pop[(long long)(base + i) * d.Np + nb.at(cx, cy, cz)] = v;
+    at(pop + (long long)(base + i) * d.Np, nb.at(cx, cy, cz)) = v;
   }
+}
+
+// push() of v and, on a z-mirror-symmetric lattice (D2), of the mirrored population, which has
+// the same value; i is the first of its pair.
+template <bool ODD, class P, int i, bool D2>
+__device__ __forceinline__ void push_pair(const Desc& d, long long cell, const Nbr& nb, int base,
+                                          P v) {
+  push<ODD, P, i>(d, cell, nb, base, v);
+  if constexpr (D2 && zmirror(i) != i) push<ODD, P, zmirror(i)>(d, cell, nb, base, v);
 }
 
 // Raw moments of a cell: rho, j = rho u, e2 = sum f|xi|^2 + sum g = 2 rho E.
@@ -148,15 +172,15 @@ struct Raw {
 };
 
 // Phase A: gather each distribution in turn and take the moments (FP64).
-template <bool ODD, class P>
+template <bool ODD, class P, bool D2 = false>
 __device__ __forceinline__ Raw gather_raw(const Desc& d, long long cell, const Nbr& nb) {
   Raw r;
   double gs;
   if constexpr (sizeof(P) == 8) {
     P h[Q];
-    gather<ODD, P>(d, cell, nb, 0, h);
+    gather<ODD, P, D2>(d, cell, nb, 0, h);
     gen::f_moments<double>(h, r.rho, r.jx, r.jy, r.jz, r.e2);
-    gather<ODD, P>(d, cell, nb, Q, h);
+    gather<ODD, P, D2>(d, cell, nb, Q, h);
     gs = gen::g_sum<double>(h);
   } else {  // deviations: moments of h_ref (precomputed) plus those of the deviations
     P h[Q];
@@ -176,10 +200,115 @@ __device__ __forceinline__ Raw gather_raw(const Desc& d, long long cell, const N
   return r;
 }
 
-template <bool ODD, class P>
+template <bool ODD, class P, bool D2 = false>
 __device__ __forceinline__ Macro gather_moments(const Desc& d, long long cell, const Nbr& nb) {
-  const Raw r = gather_raw<ODD, P>(d, cell, nb);
+  const Raw r = gather_raw<ODD, P, D2>(d, cell, nb);
   return macro_from_moments(r.rho, r.jx, r.jy, r.jz, r.e2, d.ph.inv_2cv);
+}
+
+// gather_moments out of line.
+template <bool ODD, bool D2>
+__device__ __noinline__ void gather_moments_fp64(const void* pop, long long Np, long long cell,
+                                                 const Nbr* nb, double inv_2cv, Macro* M) {
+  Desc d;
+  d.pop = const_cast<void*>(pop);
+  d.Np = Np;
+  const Raw r = gather_raw<ODD, double, D2>(d, cell, *nb);
+  *M = macro_from_moments(r.rho, r.jx, r.jy, r.jz, r.e2, inv_2cv);
+}
+
+// The macroscopic variables of a cell of a lattice one cell thick in z with the sums formed in
+// 64-bit integers: 158 FP64 additions less, each of which takes the issue time of 60 FP32
+// operations.  D2: of a z-mirror-symmetric one, with one of each mirror pair read (28 % less) and
+// the same values.
+// The populations are scaled by the power of two that brings the largest f_i into [0.25, 0.5) and
+// rounded down to units of 2^-58 (about 2^-56 of the density; the largest are exact); the sums are
+// exact.  Rounding down takes half a unit from each of the 24 populations with |xi_i|^2 >= 4 on
+// average, which is given back.  Where a population is negative, or g or the sums leave the range,
+// the cell's sums are formed in FP64.
+// On the 1024 x 512 airfoil (few solver updates) a step takes 261 us with these sums and 318 with
+// FP64 ones.  The 3-D lattices keep FP64 sums: their kernel, with the 13-multiplier solve, is bound
+// by instruction fetches, and the longer code took a step of a 128^3 box from 4.2 to 4.5 ms.
+template <bool ODD, bool D2>
+__device__ __forceinline__ Macro gather_moments_fx(const Desc& d, long long cell, const Nbr& nb) {
+  constexpr int NS = D2 ? 4 : 5;
+  fx::u64 s[NS], gs = 0;
+  int k;
+  unsigned fmax = 0, gmax = 0;
+  {
+    double f[Q];
+    gather<ODD, double, D2>(d, cell, nb, 0, f);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) fmax = max(fmax, (unsigned)__double2hiint(f[i]));
+    k = 1021 - (int)(fmax >> 20);
+    const auto val = [&](auto I) { return fx::unit58(f[decltype(I)::value], 1023 - k); };
+    if constexpr (D2) gen::macro_fx2d(val, s);
+    else gen::macro_fx(val, s);
+  }
+  {
+    double g[Q];
+    gather<ODD, double, D2>(d, cell, nb, Q, g);
+    static_for<0, Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      if constexpr (!D2 || zmirror(i) >= i) {
+        gmax = max(gmax, (unsigned)__double2hiint(g[i]));
+        const fx::u64 u = fx::unit58(g[i], 1023 - k);
+        gs += D2 && zmirror(i) != i ? 2 * u : u;
+      }
+    });
+  }
+  constexpr int E = NS - 1;
+  // scaled: f_i < 0.5 and sum f < 7, so sum f |xi|^2 < 63; g_i < 1, so sum g < 39
+  if (fmax - (100u << 20) > (1900u << 20) || gmax >= (unsigned)(1023 - k) << 20 ||
+      (unsigned)(s[0] >> 32) > (7u << 26) ||
+      ((unsigned)(s[E] >> 32) >> 1) + ((unsigned)(gs >> 32) >> 1) > (60u << 25)) {
+    const Nbr here = nb;
+    Macro M;
+    gather_moments_fp64<ODD, D2>(d.pop, d.Np, cell, &here, d.ph.inv_2cv, &M);
+    return M;
+  }
+  // products that are not contracted into the sums that follow: both systems round alike
+  const double sc = __hiloint2double((1023 - 58 - k) << 20, 0);
+  const auto value = [&](fx::u64 v) { return gen::mul_rn((double)(fx::s64)v, sc); };
+  double jz = 0.0;
+  if constexpr (!D2) jz = value(s[3]);
+  return macro_from_moments(value(s[0] + 12), value(s[1]), value(s[2]), jz,
+                            gen::mul_rn((double)(s[E] + gs + 87 + 12), sc), d.ph.inv_2cv);
+}
+
+// The same out of line, for the full system on such lattices.
+template <bool ODD>
+__device__ __noinline__ void gather_moments_thin(const void* pop, long long Np, long long cell,
+                                                 const Nbr* nb, double inv_2cv, Macro* M) {
+  Desc d;
+  d.pop = const_cast<void*>(pop);
+  d.Np = Np;
+  d.ph.inv_2cv = inv_2cv;
+  *M = gather_moments_fx<ODD, false>(d, cell, *nb);
+}
+
+// The macroscopic variables as the step of a fixed-point kernel forms them.
+template <bool ODD, bool D2>
+__device__ __forceinline__ Macro step_moments(const Desc& d, long long cell, const Nbr& nb) {
+  if constexpr (D2) return gather_moments_fx<ODD, true>(d, cell, nb);
+  if (d.nz != 1) return gather_moments<ODD, double>(d, cell, nb);
+  const Nbr here = nb;
+  Macro M;
+  gather_moments_thin<ODD>(d.pop, d.Np, cell, &here, d.ph.inv_2cv, &M);
+  return M;
+}
+
+// 39 eps in FP64 from the populations at f, where the FP32 screen cannot decide: not inlined, as
+// few cells take it (its divisions are a seventh of the step kernel's code otherwise).
+template <int BLK>
+__device__ __noinline__ double sensor_sum_fp64(const double* f, double rho, WS<BLK> F) {
+  double s = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < Q; ++i) {
+    const double feq = rho * F[i];
+    s += fabs(f[i] - feq) / feq;
+  }
+  return s;
 }
 
 // Phase C: gather again, Knudsen sensor (Eq. DeltaAvg, f only), tau_eff =
@@ -187,7 +316,7 @@ __device__ __forceinline__ Macro gather_moments(const Desc& d, long long cell, c
 // normalised equilibrium; f^eq = rho F, g^eq = (2C_v - D) T rho F.
 // PR: with the Prandtl-number adjustment (the quasi-equilibrium correction of g;
 // a separate instantiation, so the paper's Pr = 1 collision carries none of it).
-template <bool ODD, class P, int BLK, bool PR = false>
+template <bool ODD, class P, int BLK, bool PR = false, bool D2 = false>
 __device__ __forceinline__ int relax_push(const Desc& d, long long cell, const Nbr& nb,
                                           const Macro& M, WS<BLK> F) {
   const Phys& ph = d.ph;
@@ -197,45 +326,47 @@ __device__ __forceinline__ int relax_push(const Desc& d, long long cell, const N
   double eps;
   if constexpr (sizeof(P) == 8) {
     P f[Q];
-    gather<ODD, P>(d, cell, nb, 0, f);
+    gather<ODD, P, D2>(d, cell, nb, 0, f);
     // FP32 screen of 39 eps from float views (error bound: screen_undecided);
     // the FP64 value where the screen cannot decide the branch of Eq. (alpha)
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     int emin = SCREEN_EMAX, emax = SCREEN_EMIN;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double Fd = F[i];
-      const int eF = exp_field(Fd), ef = exp_field(f[i]);
-      emin = min(emin, min(eF, ef));
-      emax = max(emax, max(eF, ef));
-      const float feq = rho32 * view_float(Fd);
-      acc[i & 3] += fabsf(view_float(f[i]) - feq) * rcp32(feq);
-    }
+    static_for<0, Q>([&](auto I) {  // one of each mirror pair, counted twice
+      constexpr int i = decltype(I)::value;
+      if constexpr (!D2 || zmirror(i) >= i) {
+        const double Fd = F[i];
+        const int eF = exp_field(Fd), ef = exp_field(f[i]);
+        emin = min(emin, min(eF, ef));
+        emax = max(emax, max(eF, ef));
+        const float feq = rho32 * view_float(Fd);
+        const float t = fabsf(view_float(f[i]) - feq) * rcp32(feq);
+        acc[i & 3] += D2 && zmirror(i) != i ? 2.0f * t : t;
+      }
+    });
     const float s32 = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     eps = (double)s32 * (1.0 / Q);
     if (screen_undecided(s32, emin, emax, rho32)) {
-      double s = 0.0;
+      double fs[Q];
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const double feq = rho * F[i];
-        s += fabs(f[i] - feq) / feq;
-      }
-      eps = s * (1.0 / Q);
+      for (int i = 0; i < Q; ++i) fs[i] = f[i];
+      eps = sensor_sum_fp64<BLK>(fs, rho, F) * (1.0 / Q);
     }
     const int branch = alpha_branch(eps);
     const double omega = omega_of(ph, branch);
     static_for<0, Q>([&](auto I) {
       constexpr int i = decltype(I)::value;
-      push<ODD, P, i>(d, cell, nb, 0, fma(-omega, fma(-rho, F[i], f[i]), f[i]));
+      if constexpr (!D2 || zmirror(i) >= i)
+        push_pair<ODD, P, i, D2>(d, cell, nb, 0, fma(-omega, fma(-rho, F[i], f[i]), f[i]));
     });
     double s13[NM];
     if constexpr (PR) gen::moments_s<double>(f, s13);  // sum_i f_i phi_k(xi_i)
     P g[Q];
-    gather<ODD, P>(d, cell, nb, Q, g);
+    gather<ODD, P, D2>(d, cell, nb, Q, g);
     if constexpr (!PR) {
       static_for<0, Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        push<ODD, P, i>(d, cell, nb, Q, fma(-omega, fma(-cgr, F[i], g[i]), g[i]));
+        if constexpr (!D2 || zmirror(i) >= i)
+          push_pair<ODD, P, i, D2>(d, cell, nb, Q, fma(-omega, fma(-cgr, F[i], g[i]), g[i]));
       });
     } else {
       // heat flux q = (1/2) sum_i c_i (|c_i|^2 f_i + g_i), c_i = xi_i - u, from the raw
@@ -357,21 +488,39 @@ __device__ __forceinline__ void flush_stats(unsigned int* s_ctr, unsigned long l
 constexpr int SOLVER_PLANES = NM + Q;
 
 template <int BLK>
-__device__ __forceinline__ void load_solver_state(const Desc& d, long long cell, WS<BLK> w) {
+__device__ __forceinline__ void load_multipliers(const Desc& d, long long cell, WS<BLK> w) {
   const double* __restrict__ st = d.lam;
 #pragma unroll
-  for (int k = 0; k < NM; ++k) w[WS_LAM + k] = st[k * d.Np + cell];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) w[WS_E + i] = st[(NM + i) * d.Np + cell];
+  for (int k = 0; k < NM; ++k) w[WS_LAM + k] = at(st + k * d.Np, (int)cell);
+}
+
+template <int BLK, bool D2 = false>
+__device__ __forceinline__ void load_cached_F(const Desc& d, long long cell, WS<BLK> w) {
+  const double* __restrict__ st = d.lam;
+  static_for<0, Q>([&](auto I) {  // D2: one of each mirror pair is read
+    constexpr int i = decltype(I)::value;
+    if constexpr (!D2 || zmirror(i) >= i) {
+      const double v = at(st + (NM + i) * d.Np, (int)cell);
+      w[WS_E + i] = v;
+      if constexpr (D2 && zmirror(i) != i) w[WS_E + zmirror(i)] = v;
+    }
+  });
+}
+
+template <int BLK>
+__device__ __forceinline__ void load_solver_state(const Desc& d, long long cell, WS<BLK> w) {
+  load_multipliers<BLK>(d, cell, w);
+  load_cached_F<BLK>(d, cell, w);
 }
 
 template <int BLK>
 __device__ __forceinline__ void store_solver_state(const Desc& d, long long cell, WS<BLK> w) {
-  double* __restrict__ st = d.lam;
-#pragma unroll
-  for (int k = 0; k < NM; ++k) st[k * d.Np + cell] = w[WS_LAM + k];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) st[(NM + i) * d.Np + cell] = w[WS_E + i];
+  double* __restrict__ st = d.lam + cell;
+#pragma unroll 4
+  for (int k = 0; k < NM; ++k) st[k * d.Np] = w[WS_LAM + k];
+  st += NM * d.Np;
+#pragma unroll 4
+  for (int i = 0; i < Q; ++i) st[i * d.Np] = w[WS_E + i];
 }
 
 // F = exp(Phi lam) at the workspace multipliers.
@@ -449,14 +598,20 @@ __device__ __forceinline__ void load_solver_table() {
 // direction; 3 that after a single-precision start (start32).  The precision
 // form (P = float) always takes 3.  n32: the float steps of the start.
 // In fixed point (newton_fx) where in_fixed_point says so; a cell that it cannot
-// represent is solved again from the stored state in FP64 (newton).
+// represent is solved again from the stored state in FP64 (newton).  There the
+// workspace's multipliers are read from the stored state when the first update
+// needs them, and moved says whether the workspace's state has changed (its
+// multipliers are loaded then).
 template <class P, int BLK, bool D2, int SOLVER>
 __device__ __forceinline__ NewtonResult solve_cell(const Desc& d, long long cell, WS<BLK> w,
-                                                   const Macro& M, int maxit, int& n32) {
+                                                   const Macro& M, int maxit, int& n32,
+                                                   bool& moved) {
   constexpr bool MIXED = sizeof(P) == 4 || SOLVER >= 2, START = sizeof(P) == 4 || SOLVER == 3;
   n32 = 0;
+  moved = true;
   bool cached = true;
   if constexpr (START) {
+    if (in_fixed_point<P, SOLVER>) load_multipliers<BLK>(d, cell, w);
     if (maxit > 0) {  // a cell on the fallback off a retry step takes no step at all
       n32 = start32<BLK, D2>(w);
       cached = n32 == 0;
@@ -469,7 +624,13 @@ __device__ __forceinline__ NewtonResult solve_cell(const Desc& d, long long cell
                                      cached);
   } else {
     NewtonResult nr;
-    if (d.ph.fx && newton_fx<BLK, !MIXED, D2>(w, d.ph, maxit, cached, nr)) return nr;
+    const double* src = START ? w.p + WS_LAM * BLK : d.lam + cell;
+    if (d.ph.fx &&
+        newton_fx<BLK, !MIXED, D2>(w, src, START ? BLK : d.Np, d.ph, maxit, cached, nr, moved)) {
+      if constexpr (START) moved = moved || n32 > 0;
+      return nr;
+    }
+    moved = true;
     targets<BLK>(M.ux, M.uy, M.uz, M.T, w.at(WS_M));
     load_solver_state<BLK>(d, cell, w);
     if constexpr (START) {
@@ -490,21 +651,42 @@ __device__ __forceinline__ void step_cell(const Desc& d, long long cell, WS<BLK>
   WS<BLK> F = w.at(WS_E), lam = w.at(WS_LAM), m = w.at(WS_M);
   Coord c{0, 0, 0};
   if constexpr (ODD) c = coord_of(d, cell);
-  const Macro M = gather_moments<ODD, P>(d, cell, fresh_nbr<ODD>(d, c));
+  constexpr bool HALF = D2 && in_fixed_point<P, SOLVER>;  // one of each mirror pair is read
+  Macro M;
+  if constexpr (in_fixed_point<P, SOLVER>) M = step_moments<ODD, D2>(d, cell, fresh_nbr<ODD>(d, c));
+  else M = gather_moments<ODD, P>(d, cell, fresh_nbr<ODD>(d, c));
   targets<BLK>(M.ux, M.uy, M.uz, M.T, m);
-  load_solver_state<BLK>(d, cell, w);
-  const bool marked = is_fallback_embedding<BLK>(lam);
+  bool marked;
+  if constexpr (in_fixed_point<P, SOLVER>) {
+    load_cached_F<BLK, D2>(d, cell, w);
+    // lam_9 = -0 is the mark's first sign; the other multipliers are read only then
+    marked = __double_as_longlong(d.lam[9 * d.Np + cell]) == (long long)0x8000000000000000ull;
+    if (marked) {
+      load_multipliers<BLK>(d, cell, w);
+      marked = is_fallback_embedding<BLK>(lam);
+    }
+  } else {
+    load_solver_state<BLK>(d, cell, w);
+    marked = is_fallback_embedding<BLK>(lam);
+  }
   // a marked cell off a retry step gets no update (it stays on the fallback
   // unless its embedding already meets the 13 constraints)
   const int maxit = !marked ? d.ph.maxit : retry_budget(d.t, d.ph.maxit);
   int n32;
-  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32);
+  bool moved;
+  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32, moved);
   if (nr.failed) {
+    if (!moved) load_multipliers<BLK>(d, cell, w);
     targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // the solve may have overwritten them
     fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);
-  } else lam[9] = lam[9] + 0.0;  // a solved state carries no embedding mark
-  store_solver_state<BLK>(d, cell, w);
-  const int branch = relax_push<ODD, P, BLK, PR>(d, cell, fresh_nbr<ODD>(d, c), M, F);
+    store_solver_state<BLK>(d, cell, w);
+  } else if (moved) {
+    lam[9] = lam[9] + 0.0;  // a solved state carries no embedding mark
+    store_solver_state<BLK>(d, cell, w);
+  } else if (marked) {
+    d.lam[9 * d.Np + cell] = 0.0;
+  }
+  const int branch = relax_push<ODD, P, BLK, PR, HALF>(d, cell, fresh_nbr<ODD>(d, c), M, F);
   atomicAdd(&s_ctr[CTR_FAILED], (unsigned)nr.failed);
   atomicAdd(&s_ctr[CTR_UPDATES], (unsigned)nr.n_upd);
   atomicAdd(&s_ctr[CTR_HIST + min(nr.n_upd, 31)], 1u);
@@ -560,10 +742,11 @@ __global__ void __launch_bounds__(BLK) k_init(Desc d, const double* rho, const d
       targets<BLK>(ux, uy, uz, TT, m);
       gaussian_guess<BLK>(ux, uy, uz, TT, lam);
       NewtonResult nr;
+      [[maybe_unused]] bool moved;
       if constexpr (!in_fixed_point<P, 0>) {
         nr = newton_in<BLK, false, false>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd,
                                           maxit, false);
-      } else if (!d.ph.fx || !newton_fx<BLK, true, false>(w, d.ph, maxit, false, nr)) {
+      } else if (!d.ph.fx || !newton_fx<BLK, true, false>(w, lam.p, BLK, d.ph, maxit, false, nr, moved)) {
         targets<BLK>(ux, uy, uz, TT, m);
         gaussian_guess<BLK>(ux, uy, uz, TT, lam);
         nr = newton<BLK, false>(w, d.ph.tol, d.ph.min_upd, maxit, false);

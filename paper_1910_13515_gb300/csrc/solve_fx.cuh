@@ -10,9 +10,12 @@
 // rounding of a residual in FP64 does, and the updates a cell takes stay the
 // same.  Without it the direction is the FP32 one of root finders 2 and 3.
 //
-// What bounds it: issue slots and the latency of dependent integer and FP32
-// instructions at 12 warps an SM (an IPC of 1.8 of 4; the FP64 pipe, which bounded
-// the FP64 solve, is busy 32% with the collision).  On the 128^3 box at rms Ma 0.5 ten steps with the initialisation take 50.0 ms where the
+// What bounds it: instruction supply and the latency of dependent integer and FP32
+// instructions at 12 warps an SM (an IPC of 1.8 of 4; a fifth of the stalls wait for
+// instructions, and code that grows by a few thousand instructions costs more than
+// it saves; two blocks an SM at 255 registers without spills, and blocks of 64, 192,
+// 256 and 384 threads, with and without a barrier in each iteration, measured 2 to
+// 15 % slower).  On the 128^3 box at rms Ma 0.5 ten steps with the initialisation take 50.0 ms where the
 // FP64 solve took 259.4, on the 256^3 box at rms Ma 0.8 five take 243 where it took 1145.
 #pragma once
 #include "cell.cuh"
@@ -184,10 +187,14 @@ __device__ __forceinline__ bool multipliers_in_range(const A& l) {
   return bad == 0;
 }
 
-// The multipliers in the workspace, doubles, into units of L in place; false outside its range.
+// The multipliers at src (doubles, `stride` apart) into units of L in the workspace; false outside
+// its range.
 template <int BLK>
-__device__ __forceinline__ bool multipliers_to_log2(WS<BLK> lam) {
+__device__ __forceinline__ bool multipliers_to_log2(const double* src, long long stride,
+                                                    WS<BLK> lam) {
   const IntView<BLK> L{lam};
+#pragma unroll
+  for (int k = 0; k < NM; ++k) lam[k] = src[k * stride];
   int top = 0;
 #pragma unroll 1
   for (int k = 0; k < NM; ++k) {
@@ -198,30 +205,33 @@ __device__ __forceinline__ bool multipliers_to_log2(WS<BLK> lam) {
   return top < ((1023 + 6) << 20);
 }
 
-// The solve (see newton() for the iteration).  In: w's multipliers and targets, and with cached
-// its F at them.  Out: true with the result, w's multipliers and F (the targets are overwritten);
-// false where a value leaves the fixed-point ranges or FP32 cannot give a direction: the caller
-// restores the workspace and solves in FP64.
+// The solve (see newton() for the iteration).  In: the multipliers at src (`stride` apart: the
+// workspace's, or the stored state, which a solve that takes no update then does not read), w's
+// targets, and with cached its F at the multipliers.  Out: true with the result, w's F (the targets
+// are overwritten) and, where `moved`, its multipliers, else neither has changed; false where a
+// value leaves the fixed-point ranges or FP32 cannot give a direction: the caller restores the
+// workspace and solves in FP64.
 template <int BLK, bool REFINE, bool D2>
-__device__ __forceinline__ bool newton_fx(WS<BLK> w, const Phys& ph, int maxit, bool cached,
-                                          NewtonResult& out) {
+__device__ __forceinline__ bool newton_fx(WS<BLK> w, const double* src, long long stride,
+                                          const Phys& ph, int maxit, bool cached,
+                                          NewtonResult& out, bool& moved) {
   using S = Sys<D2>;
   constexpr int N = S::N;
   WS<BLK> F = w.at(WS_E), lam = w.at(WS_LAM), m = w.at(WS_M);
   const IntView<BLK> X{F}, L{lam}, M{m};
   int top = 0;
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const double v = m[S::idx(k)];
+  for (int k = 0; k < NM; ++k) {
+    const double v = m[k];
     top = max(top, __double2hiint(v) & 0x7fffffff);
     // rounding the 24 populations with |xi|^2 >= 4 down takes half a unit from each on average
-    const int half = S::idx(k) == 0 ? 12 : S::idx(k) >= 4 && S::idx(k) <= 6 ? 29 : 0;
-    M.set(S::idx(k), fx::signed58(v) - half);
+    const int half = k == 0 ? 12 : k >= 4 && k <= 6 ? 29 : 0;
+    M.set(k, fx::signed58(v) - half);
   }
   if (top >= (1023 + 4) << 20) return false;  // |m| >= 16, inf, NaN
   bool have_L = false;
   if (!cached) {
-    if (!multipliers_to_log2<BLK>(lam)) return false;
+    if (!multipliers_to_log2<BLK>(src, stride, lam)) return false;
     have_L = true;
   }
   int n = 0, failed = 0, ls = 0, c0 = 0;
@@ -230,7 +240,17 @@ __device__ __forceinline__ bool newton_fx(WS<BLK> w, const Phys& ph, int maxit, 
   float s0 = 0.0f;
   fx::s64 dl[N];
   for (;;) {
-    if (!(first && cached)) {
+    unsigned fmax = 0, fmin = ~0u;
+    if (first && cached) {
+#pragma unroll 1
+      for (int i = 0; i < Q; ++i) {
+        if (!D2 || ((kZOwn >> i) & 1ull)) {
+          const double v = F[i];
+          fmax = max(fmax, (unsigned)__double2hiint(v));
+          fmin = min(fmin, (unsigned)__double2hiint(v));
+        }
+      }
+    } else {
       fx::I64 l[NM], x[Q];
 #pragma unroll
       for (int k = 0; k < NM; ++k) l[k] = fx::I64(L[k]);
@@ -244,9 +264,17 @@ __device__ __forceinline__ bool newton_fx(WS<BLK> w, const Phys& ph, int maxit, 
 #pragma unroll
       for (int i = 0; i < Q; ++i) X.set(i, x[i].v);
       const fx::u64* tab = fx::table();
-#pragma unroll 1
-      for (int i = 0; i < Q; ++i)
-        if (!D2 || ((kZOwn >> i) & 1ull)) F[i] = fx::exp2_fixed(X[i], tab);
+      // three exponentials at a time from the workspace: a loop that the nearest instruction cache
+      // holds, in a kernel whose straight-line code does not fit (one at a time: 1 % slower)
+#pragma unroll 3
+      for (int i = 0; i < Q; ++i) {
+        if (!D2 || ((kZOwn >> i) & 1ull)) {
+          const double v = fx::exp2_fixed(X[i], tab);
+          F[i] = v;
+          fmax = max(fmax, (unsigned)__double2hiint(v));
+          fmin = min(fmin, (unsigned)__double2hiint(v));
+        }
+      }
       if constexpr (D2) {
         static_for<0, Q>([&](auto I) {
           constexpr int i = decltype(I)::value;
@@ -258,13 +286,7 @@ __device__ __forceinline__ bool newton_fx(WS<BLK> w, const Phys& ph, int maxit, 
     bool reject = false;
     {
       fx::u64 s[N];
-      unsigned fmax = 0, fmin = ~0u;
-      const auto val = [&](auto I) -> fx::u64 {
-        const double v = F[decltype(I)::value];
-        fmax = max(fmax, (unsigned)__double2hiint(v));
-        fmin = min(fmin, (unsigned)__double2hiint(v));
-        return fx::unit58(v);
-      };
+      const auto val = [&](auto I) { return fx::unit58(F[decltype(I)::value]); };
       if constexpr (D2) gen::sums_fx2d(val, s);
       else gen::sums_fx(val, s);
       // F_i in [2^-126, 0.75): sum F_i is below 30 and has not wrapped; below 3.5, sum F_i |xi|^2
@@ -333,7 +355,7 @@ __device__ __forceinline__ bool newton_fx(WS<BLK> w, const Phys& ph, int maxit, 
     s0 = ssq;
     c0 = c;
     if (!have_L) {
-      if (!multipliers_to_log2<BLK>(lam)) return false;
+      if (!multipliers_to_log2<BLK>(src, stride, lam)) return false;
       have_L = true;
     }
     if (!direction_fx<BLK, REFINE, D2>(F, G, b, c, dl)) return false;
@@ -342,9 +364,10 @@ __device__ __forceinline__ bool newton_fx(WS<BLK> w, const Phys& ph, int maxit, 
     ls = 0;
   }
   if (have_L) {
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < NM; ++k) lam[k] = fx::from_log2(L[k]);
   }
+  moved = have_L;
   out = NewtonResult{n, failed};
   return true;
 }

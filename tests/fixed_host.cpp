@@ -58,7 +58,9 @@ static int solve(double* ws, const Phys& ph, int maxit, int cached, int fixed, i
   WS<1> w{ws};
   NewtonResult r{-1, -1};
   if (fixed) {
-    if (!newton_fx<1, REFINE, D2>(w, ph, maxit, cached != 0, r)) return 0;
+    bool moved;
+    if (!newton_fx<1, REFINE, D2>(w, ws + WS_LAM, 1, ph, maxit, cached != 0, r, moved)) return 0;
+    out[2] = moved;
   } else {
     r = newton<1, !REFINE, D2>(w, ph.tol, ph.min_upd, maxit, cached != 0);
   }
@@ -84,7 +86,7 @@ void fx_convert(const double* F, ull* u58, const double* v, long long* s58, cons
   }
 }
 
-// One cell: ws = F (39, library order), lam (13), m (13) in; F, lam out.  Returns 0 where the
+// One cell: ws (WS_DOUBLES_FX) = F (39, library order), lam (13), m (13) in; F, lam out.  Returns 0 where the
 // fixed-point solve gives the cell up.
 int fx_solve(double* ws, int refine, int d2, int fixed, int cached, double tol, int maxit,
              int* out) {

@@ -92,7 +92,7 @@ def targets(u, T):
 
 def solve(lib, phi, lam, m, cached, refine, d2, fixed, maxit=200, tol=1e-12):
     ws = np.concatenate([np.exp(lam @ phi), lam, m])
-    out = np.zeros(2, np.int32)
+    out = np.zeros(3, np.int32)
     ok = lib.fx_solve(p(ws), refine, d2, fixed, cached, tol, maxit, p(out))
     return ok, ws[:39].copy(), ws[39:52].copy(), int(out[0]), int(out[1])
 
@@ -161,7 +161,7 @@ def test_no_update_leaves_the_multipliers_alone(lib):
     u, T = np.array([0.25, 0.1, -0.3]), 0.55
     first = solve(lib, phi, gaussian(phi, u, T), targets(u, T), 0, 1, 0, 1)
     ws = np.concatenate([first[1], first[2], targets(u, T)])
-    out = np.zeros(2, np.int32)
+    out = np.zeros(3, np.int32)
     assert lib.fx_solve(p(ws), 1, 0, 1, 1, 1e-12, 30, p(out)) == 1
-    assert out[0] == 0 and out[1] == 0
+    assert out[0] == 0 and out[1] == 0 and out[2] == 0
     assert np.array_equal(ws[:39], first[1]) and np.array_equal(ws[39:52], first[2])
