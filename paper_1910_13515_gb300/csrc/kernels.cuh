@@ -229,22 +229,20 @@ __device__ __noinline__ void gather_moments_fp64(const void* pop, long long Np, 
 // On the 1024 x 512 airfoil (few solver updates) a step takes 261 us with these sums and 318 with
 // FP64 ones.  The 3-D lattices keep FP64 sums: their kernel, with the 13-multiplier solve, is bound
 // by instruction fetches, and the longer code took a step of a 128^3 box from 4.2 to 4.5 ms.
+// f: the gathered f_i, for the caller.
 template <bool ODD, bool D2>
-__device__ __forceinline__ Macro gather_moments_fx(const Desc& d, long long cell, const Nbr& nb) {
+__device__ __forceinline__ Macro gather_moments_fx(const Desc& d, long long cell, const Nbr& nb,
+                                                   double (&f)[Q]) {
   constexpr int NS = D2 ? 4 : 5;
   fx::u64 s[NS], gs = 0;
-  int k;
   unsigned fmax = 0, gmax = 0;
-  {
-    double f[Q];
-    gather<ODD, double, D2>(d, cell, nb, 0, f);
+  gather<ODD, double, D2>(d, cell, nb, 0, f);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) fmax = max(fmax, (unsigned)__double2hiint(f[i]));
-    k = 1021 - (int)(fmax >> 20);
-    const auto val = [&](auto I) { return fx::unit58(f[decltype(I)::value], 1023 - k); };
-    if constexpr (D2) gen::macro_fx2d(val, s);
-    else gen::macro_fx(val, s);
-  }
+  for (int i = 0; i < Q; ++i) fmax = max(fmax, (unsigned)__double2hiint(f[i]));
+  const int k = 1021 - (int)(fmax >> 20);
+  const auto val = [&](auto I) { return fx::unit58(f[decltype(I)::value], 1023 - k); };
+  if constexpr (D2) gen::macro_fx2d(val, s);
+  else gen::macro_fx(val, s);
   {
     double g[Q];
     gather<ODD, double, D2>(d, cell, nb, Q, g);
@@ -284,13 +282,17 @@ __device__ __noinline__ void gather_moments_thin(const void* pop, long long Np, 
   d.pop = const_cast<void*>(pop);
   d.Np = Np;
   d.ph.inv_2cv = inv_2cv;
-  *M = gather_moments_fx<ODD, false>(d, cell, *nb);
+  double f[Q];
+  *M = gather_moments_fx<ODD, false>(d, cell, *nb, f);
 }
 
 // The macroscopic variables as the step of a fixed-point kernel forms them.
 template <bool ODD, bool D2>
 __device__ __forceinline__ Macro step_moments(const Desc& d, long long cell, const Nbr& nb) {
-  if constexpr (D2) return gather_moments_fx<ODD, true>(d, cell, nb);
+  if constexpr (D2) {
+    double f[Q];
+    return gather_moments_fx<ODD, true>(d, cell, nb, f);
+  }
   if (d.nz != 1) return gather_moments<ODD, double>(d, cell, nb);
   const Nbr here = nb;
   Macro M;
