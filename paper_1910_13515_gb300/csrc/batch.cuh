@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, 0>)) k
 
 // Boundary fills of the lattices that have freestream or outflow cells.
 template <class P>
-__global__ void k_batch_fill(const BatchEntry* __restrict__ E, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(FILL_BLK, 6) k_batch_fill(const BatchEntry* __restrict__ E, const Tile* __restrict__ tiles,
                              int s) {
   const Tile tl = tiles[blockIdx.x];
   const BatchEntry& e = E[tl.lat];
