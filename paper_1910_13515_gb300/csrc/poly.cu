@@ -20,10 +20,10 @@
 namespace lbm39 {
 namespace poly {
 
-// Threads per block of the cell kernels: FP64 issue bounds the step (two thirds of the FP64
-// operations of FP64 sums are left), and blocks of 64 fill the registers better than blocks of
-// 128: 40 steps on 2048 x 2048 take 127 ms, with 128 threads 131, with FP64 sums 151.
-constexpr int BLK = 64;
+// Threads per block of the cell kernels, and blocks an SM (168 registers): FP64 issue bounds the
+// step (two thirds of the FP64 operations of FP64 sums are left).  40 steps on 2048 x 2048 take
+// 115 ms; with 254 registers 127, with blocks of 128 threads 131, with FP64 sums 151.
+constexpr int BLK = 64, MIN_BLOCKS = 6;
 constexpr int RED_BLOCKS = 1024;  // blocks of the conserved-sum reduction
 constexpr int RED_THREADS = 128;
 
@@ -77,7 +77,7 @@ __device__ __forceinline__ void step_cell(const Desc& d, long long cell) {
 }
 
 template <bool ODD>
-__global__ void __launch_bounds__(BLK) k_poly_step(Desc d) {
+__global__ void __launch_bounds__(BLK, MIN_BLOCKS) k_poly_step(Desc d) {
   const long long cell = (long long)blockIdx.x * BLK + threadIdx.x;
   if (cell < d.N) step_cell<ODD>(d, cell);
 }
