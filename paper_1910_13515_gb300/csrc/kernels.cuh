@@ -720,11 +720,18 @@ __device__ __forceinline__ P to_store(const Desc& d, int j, double v) {
   else return __double2float_rn(v - __ldg(d.href + j));
 }
 
+// gaussian_guess out of line (39 FP64 exponentials).
+template <int BLK>
+__device__ __noinline__ void gaussian_guess_out(double ux, double uy, double uz, double T,
+                                                WS<BLK> lam) {
+  gaussian_guess<BLK>(ux, uy, uz, T, lam);
+}
+
 // Equilibrium initial condition of fluid cells in [c0, c0 + len): inputs are
 // indexed by cell - c0; u planes are `us` elements apart.  Non-fluid cells in
 // the range get zero populations and multipliers.
 template <class P, int BLK>
-__global__ void __launch_bounds__(BLK) k_init(Desc d, const double* rho, const double* u,
+__global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, 0>)) k_init(Desc d, const double* rho, const double* u,
                                               long long us, const double* T, long long c0,
                                               long long len, int maxit) {
   extern __shared__ double smem[];
@@ -743,7 +750,9 @@ __global__ void __launch_bounds__(BLK) k_init(Desc d, const double* rho, const d
       asym = uz != 0.0;
       WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M);
       targets<BLK>(ux, uy, uz, TT, m);
-      gaussian_guess<BLK>(ux, uy, uz, TT, lam);
+      bool start = false;
+      if constexpr (in_fixed_point<P, 0>) start = gaussian_guess_fx<BLK>(ux, uy, uz, TT, w);
+      if (!start) gaussian_guess_out<BLK>(ux, uy, uz, TT, lam);
       NewtonResult nr;
       [[maybe_unused]] bool moved;
       if constexpr (!in_fixed_point<P, 0>) {
@@ -751,7 +760,7 @@ __global__ void __launch_bounds__(BLK) k_init(Desc d, const double* rho, const d
                                           maxit, false);
       } else if (!d.ph.fx || !newton_fx<BLK, true, false>(w, lam.p, BLK, d.ph, maxit, false, nr, moved)) {
         targets<BLK>(ux, uy, uz, TT, m);
-        gaussian_guess<BLK>(ux, uy, uz, TT, lam);
+        gaussian_guess_out<BLK>(ux, uy, uz, TT, lam);
         nr = newton<BLK, false>(w, d.ph.tol, d.ph.min_upd, maxit, false);
       }
       if (nr.failed) {
