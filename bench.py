@@ -90,12 +90,12 @@ NCU_TRAFFIC = {"kernel_hash": "98f81eefb40860d3",
                                  "box384/mixed": 82.86}}
 # The sources the step kernels and their launches are built from (the serving-form kernels
 # in batch.cuh are not among them).
-KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "kernels.cuh",
-                  "lbm39.cu")
+KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
+                  "kernels.cuh", "launch.cuh", "solve_fx.cuh", "lbm39.cu")
 # The same for the polynomial comparison model's step kernel, and its ncu DRAM bytes per
 # launch (per lattice side n of the n x n x 1 workload; null once the code differs).
-POLY_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "kernels.cuh",
-                "poly_eq.cuh", "poly.cu")
+POLY_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
+                "kernels.cuh", "solve_fx.cuh", "poly_eq.cuh", "poly.cu")
 POLY_NCU_TRAFFIC = {"kernel_hash": "02dc9070eca147c2",
                     # 2048: the 1024 capture scaled by the cell count (both exceed L2)
                     "gb_per_launch": {"1024": 1.272, "2048": 5.087}}

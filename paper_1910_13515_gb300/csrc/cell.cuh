@@ -4,12 +4,14 @@
 // not fit in registers live in shared memory with a stride of the block size
 // (WS), so a warp touches 32 consecutive doubles and hits no bank conflict.
 //
-// The GB300 issues FP64 at about 1/64 of the FP32 rate, so the FP64 step is
-// bound by its FP64 operation count.  The sums over the 39 velocities come
-// from gen_d3q39.py (sign-orbit butterflies: the same sums, reorganised), the
-// exponential is exp_tang (9 FP64 operations), and the Knudsen sensor is
-// screened in FP32 and recomputed in FP64 only near a threshold of Eq. (alpha),
-// so alpha is the one an FP64 evaluation gives.
+// The GB300 issues FP64 at about 1/60 of the FP32 rate.  The FP64 path's constraint
+// solve therefore runs in fixed point on the integer and FP32 pipes (fixed.cuh,
+// solve_fx.cuh); what is here in FP64 is the solve of the precision form and of the
+// chord-Newton hybrid, and of the cells that fixed point cannot represent.  Their
+// sums over the 39 velocities come from gen_d3q39.py (sign-orbit butterflies: the
+// same sums, reorganised), the exponential is exp_tang (9 FP64 operations), and the
+// Knudsen sensor is screened in FP32 and recomputed in FP64 only near a threshold of
+// Eq. (alpha), so alpha is the one an FP64 evaluation gives.
 #pragma once
 #include <cmath>
 
