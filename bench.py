@@ -79,15 +79,16 @@ FP64_FLOPS_MODEL = {
     # 128^3 box at rms Ma 0.8 (2.003 updates, every solve started: 3552 flops per cell) and
     # 0.3 (1.982: 3526)
     "fp64_fp32start": (691.0, 1047.0, 761.0)}
-# DRAM bytes (read + write) per launch of the step kernel from ncu, per workload and
-# precision, with the hash of the step kernel's code they were captured with; reported as
-# null once that code differs (profiles/ has the captures).  The 256^3 and 384^3 figures are
-# the 128^3 captures scaled by the cell count (x 8, x 27; the same per-cell work, all far
-# beyond L2).
-NCU_TRAFFIC = {"kernel_hash": "98f81eefb40860d3",
-               "gb_per_launch": {"box128/fp64": 4.705, "box256/fp64": 37.64,
-                                 "box128/mixed": 3.069, "box256/mixed": 24.55,
-                                 "box384/mixed": 82.86}}
+# DRAM bytes (read + write) and warp instructions (smsp__inst_executed) per launch of the step
+# kernel from ncu, mean of an even and an odd launch, per workload and precision, with the hash
+# of the step kernel's code they were captured with; reported as null once that code differs
+# (profiles/k_step_fixed_point.md has the captures).  The 256^3 figures are the 128^3 captures
+# scaled by the cell count (x 8; the same per-cell work, both far beyond L2; a warp takes the
+# updates of its slowest cell, so the count hardly depends on the mean of its cells).
+NCU_LAUNCH = {"kernel_hash": "f4c0d3664027b73e",
+              "gb": {"box128/fp64": 6.77, "box256/fp64": 54.2, "naca/fp64": 2.88},
+              "warp_instructions": {"box128/fp64": 2.416e9, "box256/fp64": 19.33e9,
+                                    "naca/fp64": 0.3237e9}}
 # The sources the step kernels and their launches are built from (the serving-form kernels
 # in batch.cuh are not among them).
 KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
@@ -96,9 +97,9 @@ KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.c
 # launch (per lattice side n of the n x n x 1 workload; null once the code differs).
 POLY_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
                 "kernels.cuh", "solve_fx.cuh", "poly_eq.cuh", "poly.cu")
-POLY_NCU_TRAFFIC = {"kernel_hash": "02dc9070eca147c2",
-                    # 2048: the 1024 capture scaled by the cell count (both exceed L2)
-                    "gb_per_launch": {"1024": 1.272, "2048": 5.087}}
+POLY_NCU_TRAFFIC = {"kernel_hash": "6e164d1b83de7ee2",
+                    # 2048: mean of an even (5.22) and an odd launch (8.04: it spills)
+                    "gb_per_launch": {"2048": 6.63}}
 
 
 def source_code_text(text: str) -> str:
@@ -118,9 +119,10 @@ def kernel_source_hash(sources=KERNEL_SOURCES) -> str:
         h.update(b"\0")
     return h.hexdigest()[:16]
 # FP64 flops of one cell update of the polynomial comparison model, counted from its source
-# (2 per FMA, identical subexpressions once): moments 120, sum g 38, rho/u/T 21, cell
-# coefficients 35, shell coefficients 70, rest velocity 7, xi.u 32, 19 (xi, -xi) pairs x 20.
-POLY_FLOPS_PER_UPDATE = 703
+# (2 per FMA, identical subexpressions once): rho/u/T 21, cell coefficients 35, shell
+# coefficients 70, rest velocity 7, xi.u 32, 19 (xi, -xi) pairs x 20.  The moments and sum g
+# (158 operations) are integer sums.
+POLY_FLOPS_PER_UPDATE = 545
 # populations read + written, and the per-cell solver state (lam and F: 52 FP64) read + written
 BYTES_PER_UPDATE = {"fp64": 78 * 8 * 2 + 52 * 8 * 2, "mixed": 78 * 4 * 2 + 52 * 8 * 2}
 
@@ -419,7 +421,7 @@ def run_serve(args, rank, world, local):
 def run_poly(args, rank, world, local):
     """The polynomial-equilibrium comparison model on the paper's comparison size: value =
     MLUPS of lbm39_poly_step (device-timed), roofline against the FP64 pipe (the binding one at
-    703 flops and 1248 bytes per update), e2e through PolyLattice with host buffers."""
+    545 flops and 1248 bytes per update), e2e through PolyLattice with host buffers."""
     import numpy as np
     import torch
     import torch.distributed as dist
@@ -905,10 +907,12 @@ def main():
                   if model else None)
     achieved_tf = flops_cell * fluid / (step_ms * 1e-3) / 1e12 if model else None
     hbm_gbs = BYTES_PER_UPDATE[args.precision] * fluid / (step_ms * 1e-3) / 1e9
-    traffic = None
-    if (NCU_TRAFFIC["kernel_hash"] == kernel_source_hash() and args.mach == 0.8
-            and args.root_finder == "newton" and args.newton_tol == 1e-12):
-        traffic = NCU_TRAFFIC["gb_per_launch"].get(f"{args.workload}/{args.precision}")
+    traffic = issue = None
+    if (NCU_LAUNCH["kernel_hash"] == kernel_source_hash() and args.mach == 0.8
+            and args.root_finder == "newton" and args.newton_tol == 1e-12
+            and not args.start_at and not args.checkpoint_in):
+        traffic = NCU_LAUNCH["gb"].get(f"{args.workload}/{args.precision}")
+        issue = NCU_LAUNCH["warp_instructions"].get(f"{args.workload}/{args.precision}")
     roofline = {"bound": "alu", "achieved": round(achieved_tf, 4) if model else None,
                 "peak": round(peak_tf, 4), "unit": "TFLOP/s",
                 "frac": round(achieved_tf / peak_tf, 4) if model else None,
@@ -925,6 +929,24 @@ def main():
                         "frac": round(hbm_gbs / HBM_PEAK_GBS, 4),
                         "bytes_per_update": BYTES_PER_UPDATE[args.precision],
                         "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)"}}
+
+    if args.precision == "fp64" and args.root_finder != "chord":
+        # these kernels solve in fixed point: the FP64 flops of the model are the formulation's
+        # and not executed, and the issue slots (4 warp instructions per clock and SM) bound
+        sms = torch.cuda.get_device_properties(local).multi_processor_count
+        peak = 4 * sms * (clocks["sm_mhz"] or clocks["sm_max_mhz"] or 2070.0) * 1e6 / 1e9
+        rate = issue / (step_ms * 1e-3) / 1e9 if issue else None
+        roofline = {"bound": "issue", "achieved": round(rate, 1) if issue else None,
+                    "peak": round(peak, 1), "unit": "Gwarp-instructions/s",
+                    "frac": round(rate / peak, 4) if issue else None,
+                    "traffic": roofline["traffic"],
+                    "peak_source": "4 warp instructions per clock and SM at the SM clock sampled "
+                                   "in this run",
+                    "instructions_per_launch": issue,
+                    "fp64_formulation": {"flops_per_cell_update": roofline["flops_per_cell_update"],
+                                         "equivalent_tflops": roofline["achieved"],
+                                         "fp64_peak_tflops": roofline["peak"]},
+                    "hbm": roofline["hbm"]}
 
     # end to end through the C ABI with host buffers: upload the initial fields from pinned
     # memory, then every step a step and a read-back of rho/u/T/p into pinned memory
