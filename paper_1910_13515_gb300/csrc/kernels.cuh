@@ -26,6 +26,7 @@
 
 #include "cell.cuh"
 #include "launch.cuh"
+#include "plane.cuh"
 #include "solve_fx.cuh"
 
 namespace lbm39 {
@@ -106,16 +107,6 @@ __device__ __forceinline__ Nbr fresh_nbr(const Desc& d, Coord c) {
     nb = Nbr(d, c);
   }
   return nb;
-}
-
-// Element at an index of a plane.  The plane's address is the same for all threads, and the byte
-// offset in it fits in 32 bits (a plane of 2^32 bytes is one of 2^29 doubles, and the 130 planes of
-// such a lattice are twice the memory of a GB300): one instruction with a uniform base and a 32-bit
-// offset, where 64-bit addresses took ten for each of a cell's 300 accesses.
-template <class P>
-__device__ __forceinline__ P& at(P* plane, int index) {
-  return *reinterpret_cast<P*>(reinterpret_cast<char*>(const_cast<std::remove_const_t<P>*>(plane)) +
-                               (unsigned)index * (unsigned)sizeof(P));
 }
 
 // Pre-collision populations of one distribution (base 0: f, Q: g) of fluid
