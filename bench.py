@@ -92,11 +92,11 @@ NCU_LAUNCH = {"kernel_hash": "f4c0d3664027b73e",
 # The sources the step kernels and their launches are built from (the serving-form kernels
 # in batch.cuh are not among them).
 KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
-                  "kernels.cuh", "launch.cuh", "solve_fx.cuh", "lbm39.cu")
+                  "kernels.cuh", "launch.cuh", "plane.cuh", "solve_fx.cuh", "lbm39.cu")
 # The same for the polynomial comparison model's step kernel, and its ncu DRAM bytes per
 # launch (per lattice side n of the n x n x 1 workload; null once the code differs).
 POLY_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
-                "kernels.cuh", "solve_fx.cuh", "poly_eq.cuh", "poly.cu")
+                "kernels.cuh", "plane.cuh", "solve_fx.cuh", "poly_eq.cuh", "poly.cu")
 POLY_NCU_TRAFFIC = {"kernel_hash": "6e164d1b83de7ee2",
                     # 2048: mean of an even (5.22) and an odd launch (8.04: it spills)
                     "gb_per_launch": {"2048": 6.63}}
@@ -971,7 +971,10 @@ def main():
                "steps": ke, "includes": "lbm39_init_host once (cold-start Newton) + per step "
                                        "lbm39_step(1) and lbm39_read_host of rho,u,T,p"}
         del h_rho, h_u, h_T, h_out
-    launches = args.steps * (2 if L.has_fills else 1)
+    # a step of the fixed-point form is two launches: its kernel, and the FP64 kernel for what that
+    # left
+    two = prec == C.LBM39_FP64 and L.params.root_finder != 1 and L.params.newton_tol >= 2e-13
+    launches = args.steps * (1 + int(two) + int(L.has_fills))
 
     # precision form against the FP64 path on the same input and step count (single run)
     form = None

@@ -77,7 +77,10 @@ typedef struct {
   double gamma;             /* heat-capacity ratio, C_v = 1/(gamma-1) (Sec. 2); > 1 */
   double tau;               /* BGK relaxation time tau_f = tau_g (Pr = 1); >= 0.5 */
   int32_t kn_sensor;        /* 1: tau(eps) = tau*alpha(eps) (Eq. alpha); 0: plain BGK */
-  double newton_tol;        /* stop when max_k |G_k|/rho < tol (Sec. 5); default 1e-12 */
+  double newton_tol;        /* stop when max_k |G_k|/rho < tol (Sec. 5); default 1e-12.
+                               From 2e-13 to 1 the FP64 path solves in 64-bit fixed point;
+                               below and above, and in cells outside its ranges, in FP64,
+                               which takes about five times as long. */
   int32_t newton_maxit;     /* updates per solve before a cell counts as failed; 30 */
   int32_t newton_min_upd;   /* updates taken even from a converged warm start; 0 */
   int32_t init_maxit;       /* cold-start updates allowed in lbm39_init; 200 */

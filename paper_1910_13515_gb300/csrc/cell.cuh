@@ -450,8 +450,8 @@ __device__ __forceinline__ NewtonResult newton_in(WS<BLK> w, DL dl, const double
   return NewtonResult{n, failed};
 }
 
-// The solve of the cells outside the ranges of newton_fx, and of single states: not inlined, as
-// few cells take it, its direction on the stack.
+// The solve of single states and, in the diagnostic fields, of the cells outside the ranges of
+// newton_fx: not inlined, as few cells take it, its direction on the stack.
 template <int BLK, bool MIXED, bool D2 = false>
 __device__ __noinline__ NewtonResult newton(WS<BLK> w, double tol, int min_upd, int maxit,
                                             bool cached) {

@@ -40,6 +40,19 @@ __device__ __forceinline__ Macro moments_of(const Desc& d, long long cell) {
   else return gather_moments<ODD, P>(d, cell, nb);
 }
 
+// The FP64 solve of a cell that newton_fx gave up, from the stored state.
+template <int BLK, bool D2, int SOLVER>
+__device__ __forceinline__ NewtonResult solve_again(const Desc& d, long long cell, WS<BLK> w,
+                                                    const Macro& M, int maxit, int& n32) {
+  targets<BLK>(M.ux, M.uy, M.uz, M.T, w.at(WS_M));
+  load_solver_state<BLK>(d, cell, w);
+  n32 = 0;
+  if constexpr (SOLVER == 3) {
+    if (maxit > 0) n32 = start32<BLK, D2>(w);
+  }
+  return newton<BLK, (SOLVER >= 2), D2>(w, d.ph.tol, d.ph.min_upd, maxit, n32 == 0);
+}
+
 // eps: FP64 (1/Q) sum_i |f_i - f_i^eq| / f_i^eq of the state against the
 // equilibrium the next step relaxes to; n_upd: its Newton updates, -1 where
 // the solve fails (the cell takes the fallback equilibrium).  Non-fluid cells
@@ -68,7 +81,12 @@ __global__ void __launch_bounds__(solve_blk(in_fixed_point<P, SOLVER>))
   const int maxit = !marked ? d.ph.maxit : retry_budget(d.t, d.ph.maxit);
   int n32;
   bool moved;
-  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32, moved);
+  NewtonResult nr;
+  bool solved = false;
+  if (!FIXED || d.ph.fx) solved = solve_cell<P, BLK, D2, SOLVER, FIXED>(d, cell, w, maxit, nr, n32, moved);
+  if constexpr (FIXED) {
+    if (!solved) nr = solve_again<BLK, D2, SOLVER>(d, cell, w, M, maxit, n32);
+  }
   if (nr.failed) {
     targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // the solve may have overwritten them
     fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);

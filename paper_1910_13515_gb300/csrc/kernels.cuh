@@ -31,10 +31,17 @@
 
 namespace lbm39 {
 
+// Cells of one warp: 32 w + the bits that are set.
+struct Rest {
+  unsigned w, bits;
+};
+
 struct Desc {
   void* pop;                          // 78 planes of P
   double* lam;                        // 13 planes of multipliers kept between steps, then
                                       // 39 planes of F_i = exp(Phi lam) at them
+  Rest* rest;                         // the cells that a fixed-point kernel leaves to its FP64
+                                      // kernel (k_step_fp64, k_init_fp64)
   const uint8_t* mask;                // nullptr: every cell fluid, all axes periodic
   unsigned long long* ctr;            // counters (CTR_*)
   const void* free_store;             // 78 stored values (P) of a freestream cell
@@ -57,6 +64,11 @@ enum {
 // Set by lbm39_init when some fluid cell starts with u_z != 0 (outside the
 // block counters: not reported by lbm39_stats).
 constexpr int CTR_ASYM = 42;
+// Lengths of the lists of cells left to the FP64 kernels, also outside the block counters: steps at
+// even and odd times, then alternate ranges of an initialisation.  A list's length is zero before
+// its fixed-point kernel, since the FP64 kernel that follows one list clears the other of its pair.
+// CTR_TAKEN: the entries of each that the FP64 kernel's warps took beyond their first.
+constexpr int CTR_REST = 44, CTR_TAKEN = 48;
 
 struct Coord {
   int x, y, z;
@@ -590,48 +602,37 @@ __device__ __forceinline__ void load_solver_table() {
 // 1 the chord-Newton hybrid (newton_chord); 2 Newton with a single-precision
 // direction; 3 that after a single-precision start (start32).  The precision
 // form (P = float) always takes 3.  n32: the float steps of the start.
-// In fixed point (newton_fx) where in_fixed_point says so; a cell that it cannot
-// represent is solved again from the stored state in FP64 (newton).  There the
+// FIXED: in fixed point (newton_fx); false for a cell that it cannot represent,
+// whose stored state has not changed: it is solved in FP64.  There the
 // workspace's multipliers are read from the stored state when the first update
 // needs them, and moved says whether the workspace's state has changed (its
-// multipliers are loaded then).
-template <class P, int BLK, bool D2, int SOLVER>
-__device__ __forceinline__ NewtonResult solve_cell(const Desc& d, long long cell, WS<BLK> w,
-                                                   const Macro& M, int maxit, int& n32,
-                                                   bool& moved) {
+// multipliers are loaded then).  Else in FP64, always true.
+template <class P, int BLK, bool D2, int SOLVER, bool FIXED>
+__device__ __forceinline__ bool solve_cell(const Desc& d, long long cell, WS<BLK> w, int maxit,
+                                           NewtonResult& nr, int& n32, bool& moved) {
   constexpr bool MIXED = sizeof(P) == 4 || SOLVER >= 2, START = sizeof(P) == 4 || SOLVER == 3;
   n32 = 0;
   moved = true;
   bool cached = true;
   if constexpr (START) {
-    if (in_fixed_point<P, SOLVER>) load_multipliers<BLK>(d, cell, w);
+    if (FIXED) load_multipliers<BLK>(d, cell, w);
     if (maxit > 0) {  // a cell on the fallback off a retry step takes no step at all
       n32 = start32<BLK, D2>(w);
       cached = n32 == 0;
     }
   }
-  if constexpr (!in_fixed_point<P, SOLVER>) {
-    if constexpr (SOLVER == 1 && sizeof(P) == 8)
-      return newton_chord<BLK, D2>(w, d.ph, maxit, true);
-    else
-      return newton_in<BLK, MIXED, D2>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd, maxit,
-                                       cached);
-  } else {
-    NewtonResult nr;
+  if constexpr (FIXED) {
     const double* src = START ? w.p + WS_LAM * BLK : d.lam + cell;
-    if (d.ph.fx &&
-        newton_fx<BLK, !MIXED, D2>(w, src, START ? BLK : d.Np, d.ph, maxit, cached, nr, moved)) {
-      if constexpr (START) moved = moved || n32 > 0;
-      return nr;
-    }
-    moved = true;
-    targets<BLK>(M.ux, M.uy, M.uz, M.T, w.at(WS_M));
-    load_solver_state<BLK>(d, cell, w);
-    if constexpr (START) {
-      if (maxit > 0) start32<BLK, D2>(w);  // as above: the same cached
-    }
-    return newton<BLK, MIXED, D2>(w, d.ph.tol, d.ph.min_upd, maxit, cached);
+    if (!newton_fx<BLK, !MIXED, D2>(w, src, START ? BLK : d.Np, d.ph, maxit, cached, nr, moved))
+      return false;
+    if constexpr (START) moved = moved || n32 > 0;
+  } else if constexpr (SOLVER == 1 && sizeof(P) == 8) {
+    nr = newton_chord<BLK, D2>(w, d.ph, maxit, true);
+  } else {
+    nr = newton_in<BLK, MIXED, D2>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd, maxit,
+                                   cached);
   }
+  return true;
 }
 
 // One fluid cell's time step (even or odd AA pass): phases A, B and C, with
@@ -639,19 +640,23 @@ __device__ __forceinline__ NewtonResult solve_cell(const Desc& d, long long cell
 // D2: the nine-function constraint system of a z-mirror-symmetric lattice one
 // cell thick in z (Sys<true>; the same values as the full system).
 // SOLVER: the root finder of the constraint equations (solve_cell).
-template <bool ODD, class P, int BLK, bool D2 = false, bool PR = false, int SOLVER = 0>
-__device__ __forceinline__ void step_cell(const Desc& d, long long cell, WS<BLK> w,
+// FIXED: solved in fixed point; true, with nothing done, for a cell that is left
+// to the FP64 step.
+template <bool ODD, class P, int BLK, bool D2 = false, bool PR = false, int SOLVER = 0,
+          bool FIXED = in_fixed_point<P, SOLVER>>
+__device__ __forceinline__ bool step_cell(const Desc& d, long long cell, WS<BLK> w,
                                           unsigned int* s_ctr) {
   WS<BLK> F = w.at(WS_E), lam = w.at(WS_LAM), m = w.at(WS_M);
   Coord c{0, 0, 0};
   if constexpr (ODD) c = coord_of(d, cell);
-  constexpr bool HALF = D2 && in_fixed_point<P, SOLVER>;  // one of each mirror pair is read
+  constexpr bool INTEGER = in_fixed_point<P, SOLVER>;  // also in the FP64 step of such a lattice
+  constexpr bool HALF = D2 && INTEGER;                 // one of each mirror pair is read
   Macro M;
-  if constexpr (in_fixed_point<P, SOLVER>) M = step_moments<ODD, D2>(d, cell, fresh_nbr<ODD>(d, c));
+  if constexpr (INTEGER) M = step_moments<ODD, D2>(d, cell, fresh_nbr<ODD>(d, c));
   else M = gather_moments<ODD, P>(d, cell, fresh_nbr<ODD>(d, c));
   targets<BLK>(M.ux, M.uy, M.uz, M.T, m);
   bool marked;
-  if constexpr (in_fixed_point<P, SOLVER>) {
+  if constexpr (FIXED) {
     load_cached_F<BLK, D2>(d, cell, w);
     // lam_9 = -0 is the mark's first sign; the other multipliers are read only then
     marked = __double_as_longlong(d.lam[9 * d.Np + cell]) == (long long)0x8000000000000000ull;
@@ -668,10 +673,18 @@ __device__ __forceinline__ void step_cell(const Desc& d, long long cell, WS<BLK>
   const int maxit = !marked ? d.ph.maxit : retry_budget(d.t, d.ph.maxit);
   int n32;
   bool moved;
-  const NewtonResult nr = solve_cell<P, BLK, D2, SOLVER>(d, cell, w, M, maxit, n32, moved);
+  NewtonResult nr;
+  const unsigned lanes = __activemask();
+  const bool solved = solve_cell<P, BLK, D2, SOLVER, FIXED>(d, cell, w, maxit, nr, n32, moved);
+  if constexpr (FIXED) {
+    // the lanes go on together: with the return below, the compiler otherwise left a warp as its
+    // solves had diverged, and phase C ran 1.7 times for each (a 128^3 box 54 ms, not 44.5)
+    __syncwarp(lanes);
+    if (!solved) return true;
+  }
   if (nr.failed) {
     if (!moved) load_multipliers<BLK>(d, cell, w);
-    targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // the solve may have overwritten them
+    if constexpr (FIXED) targets<BLK>(M.ux, M.uy, M.uz, M.T, m);  // newton_fx overwrites them
     fallback_cell<BLK>(d.lam, d.Np, cell, w, M.T, marked);
     store_solver_state<BLK>(d, cell, w);
   } else if (moved) {
@@ -689,6 +702,50 @@ __device__ __forceinline__ void step_cell(const Desc& d, long long cell, WS<BLK>
     atomicAdd(&s_ctr[CTR_UPD32], (unsigned)n32);
     atomicAdd(&s_ctr[CTR_START32], 1u);
   }
+  return false;
+}
+
+// The cells that a fixed-point kernel leaves to the FP64 solve.  They are few, but one of them can
+// take hundreds of evaluations, and the slowest ends the step; they come in clusters, and the four
+// warps of a block, solving in FP64 where they are, share one SM's FP64 pipe.  So the whole step of
+// such a cell is put off to a launch of its own (its slots of the AA buffer are its own), whose
+// warps take the list's entries one by one and which has the 255 registers of an FP64 solve.
+// A 64^3 box at rms Ma 1.3 takes 136 ms for 8 steps; with these cells solved in place, at the
+// fixed-point kernel's 168 registers, 196, and with FP64 solves for all cells 161.
+// leave: by whole warps; appends the cells of the lanes with left set to list k.
+__device__ __forceinline__ void leave(const Desc& d, int k, long long cell, bool left) {
+  const unsigned bits = __ballot_sync(0xffffffffu, left);
+  if (bits != 0 && (threadIdx.x & 31) == 0)
+    d.rest[atomicAdd(d.ctr + CTR_REST + k, 1ull)] = Rest{(unsigned)(cell >> 5), bits};
+}
+
+// The entry that this warp takes after entry e, of lists shared by `warps` warps.
+__device__ __forceinline__ long long next_entry(unsigned long long* taken, long long warps) {
+  unsigned long long e = 0;
+  if ((threadIdx.x & 31) == 0) e = atomicAdd(taken, 1ull);
+  return warps + (long long)__shfl_sync(0xffffffffu, e, 0);
+}
+
+// Calls f(cell) for each cell of list k, or with all for each of n cells; a warp takes the 32 cells
+// of an entry together, as the fixed-point kernel had them.
+template <class F>
+__device__ __forceinline__ void for_rest(const Desc& d, int k, bool all, long long n, F&& f) {
+  const long long warps = (long long)gridDim.x * (blockDim.x / 32);
+  const long long count = all ? (n + 31) / 32 : (long long)d.ctr[CTR_REST + k];
+  long long e = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  while (e < count) {
+    const Rest r = all ? Rest{(unsigned)e, 0xffffffffu} : d.rest[e];
+    const long long cell = (long long)r.w * 32 + (threadIdx.x & 31);
+    if ((r.bits >> (threadIdx.x & 31) & 1) && cell < n) f(cell);
+    __syncwarp();
+    e = all ? count : next_entry(d.ctr + CTR_TAKEN + k, warps);
+  }
+}
+
+// Empties list k before its next use.
+__device__ __forceinline__ void clear_rest(const Desc& d, int k) {
+  d.ctr[CTR_REST + k] = 0;
+  d.ctr[CTR_TAKEN + k] = 0;
 }
 
 // One time step over every fluid cell (even or odd AA pass).
@@ -699,8 +756,32 @@ __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, SOLVER
   for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
   load_solver_table<in_fixed_point<P, SOLVER>>();
   const long long cell = (long long)blockIdx.x * BLK + threadIdx.x;
+  bool left = false;
   if (cell < d.N && (d.mask == nullptr || d.mask[cell] == MASK_FLUID))
-    step_cell<ODD, P, BLK, D2, PR, SOLVER>(d, cell, WS<BLK>{smem + threadIdx.x}, s_ctr);
+    left = step_cell<ODD, P, BLK, D2, PR, SOLVER>(d, cell, WS<BLK>{smem + threadIdx.x}, s_ctr);
+  if constexpr (in_fixed_point<P, SOLVER>) leave(d, ODD, cell, left);
+  flush_stats<BLK>(s_ctr, d.ctr);
+}
+
+// The step of the cells left by k_step, or with all of every fluid cell, solved in FP64.  All: the
+// lattices whose tolerance is below the fixed-point resolution (at 1e-13 a 64^3 box's 8 steps take
+// 24.6 ms; 25.4 where the fixed-point kernel called the FP64 solve for each cell).
+template <bool ODD, bool D2, bool PR, int SOLVER>
+__global__ void __launch_bounds__(solve_blk(false), solve_min_blocks(false))
+    k_step_fp64(Desc d, bool all) {
+  constexpr int BLK = solve_blk(false);
+  extern __shared__ double smem[];
+  __shared__ unsigned int s_ctr[CTR_N];
+  cudaGridDependencySynchronize();
+  if (blockIdx.x == 0 && threadIdx.x == 0) clear_rest(d, !ODD);
+  if (!all && d.ctr[CTR_REST + ODD] == 0) return;
+  for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
+  load_exp_table();
+  for_rest(d, ODD, all, d.N, [&](long long cell) {
+    if (d.mask == nullptr || d.mask[cell] == MASK_FLUID)
+      step_cell<ODD, double, BLK, D2, PR, SOLVER, false>(d, cell, WS<BLK>{smem + threadIdx.x},
+                                                         s_ctr);
+  });
   flush_stats<BLK>(s_ctr, d.ctr);
 }
 
@@ -718,59 +799,92 @@ __device__ __noinline__ void gaussian_guess_out(double ux, double uy, double uz,
   gaussian_guess<BLK>(ux, uy, uz, T, lam);
 }
 
-// Equilibrium initial condition of fluid cells in [c0, c0 + len): inputs are
+// Equilibrium initial condition of a cell, its inputs at index r; returns whether it is left to
+// the FP64 kernel (FIXED; nothing is written then).  asym: whether it starts with u_z != 0.
+template <class P, int BLK, bool FIXED>
+__device__ __forceinline__ bool init_cell(const Desc& d, const double* rho, const double* u,
+                                          long long us, const double* T, long long cell,
+                                          long long r, int maxit, WS<BLK> w, unsigned int* s_ctr,
+                                          bool& asym) {
+  P* pop = static_cast<P*>(d.pop);
+  if (d.mask != nullptr && d.mask[cell] != MASK_FLUID) {
+    for (int j = 0; j < 2 * Q; ++j) pop[(long long)j * d.Np + cell] = P(0);
+    for (int k = 0; k < SOLVER_PLANES; ++k) d.lam[k * d.Np + cell] = 0.0;
+    return false;
+  }
+  const double rr = rho[r], ux = u[r], uy = u[us + r], uz = u[2 * us + r], TT = T[r];
+  asym = uz != 0.0;
+  WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M);
+  targets<BLK>(ux, uy, uz, TT, m);
+  NewtonResult nr;
+  if constexpr (FIXED) {
+    bool moved;
+    const unsigned lanes = __activemask();
+    const bool solved = gaussian_guess_fx<BLK>(ux, uy, uz, TT, w) &&
+                        newton_fx<BLK, true, false>(w, lam.p, BLK, d.ph, maxit, false, nr, moved);
+    __syncwarp(lanes);  // as in step_cell
+    if (!solved) return true;
+    if (nr.failed) targets<BLK>(ux, uy, uz, TT, m);  // newton_fx overwrites them
+  } else {
+    gaussian_guess_out<BLK>(ux, uy, uz, TT, lam);
+    nr = newton_in<BLK, false, false>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd, maxit,
+                                      false);
+  }
+  if (nr.failed) fallback_cell<BLK>(d.lam, d.Np, cell, w, TT, false);
+  store_solver_state<BLK>(d, cell, w);
+  const double cgr = d.ph.cg * TT * rr;
+  for (int i = 0; i < Q; ++i) {
+    pop[(long long)i * d.Np + cell] = to_store<P>(d, i, rr * F[i]);
+    pop[(long long)(Q + i) * d.Np + cell] = to_store<P>(d, Q + i, cgr * F[i]);
+  }
+  atomicAdd(&s_ctr[CTR_FAILED], (unsigned)nr.failed);
+  return false;
+}
+
+// Equilibrium initial condition of the cells in [c0, c0 + len): inputs are
 // indexed by cell - c0; u planes are `us` elements apart.  Non-fluid cells in
-// the range get zero populations and multipliers.
+// the range get zero populations and multipliers.  list: where the cells left
+// to the FP64 kernel go.
 template <class P, int BLK>
 __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, 0>)) k_init(Desc d, const double* rho, const double* u,
                                               long long us, const double* T, long long c0,
-                                              long long len, int maxit) {
+                                              long long len, int maxit, int list) {
+  constexpr bool FIXED = in_fixed_point<P, 0>;
   extern __shared__ double smem[];
   __shared__ unsigned int s_ctr[CTR_N];
   for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
-  load_solver_table<in_fixed_point<P, 0>>();
+  load_solver_table<FIXED>();
   const long long r = (long long)blockIdx.x * BLK + threadIdx.x;
-  const long long cell = c0 + r;
-  P* pop = static_cast<P*>(d.pop);
-  int asym = 0;
-  if (r < len && cell < d.N) {
-    const bool fluid = d.mask == nullptr || d.mask[cell] == MASK_FLUID;
-    WS<BLK> w{smem + threadIdx.x};
-    if (fluid) {
-      const double rr = rho[r], ux = u[r], uy = u[us + r], uz = u[2 * us + r], TT = T[r];
-      asym = uz != 0.0;
-      WS<BLK> lam = w.at(WS_LAM), F = w.at(WS_E), m = w.at(WS_M);
-      targets<BLK>(ux, uy, uz, TT, m);
-      bool start = false;
-      if constexpr (in_fixed_point<P, 0>) start = gaussian_guess_fx<BLK>(ux, uy, uz, TT, w);
-      if (!start) gaussian_guess_out<BLK>(ux, uy, uz, TT, lam);
-      NewtonResult nr;
-      [[maybe_unused]] bool moved;
-      if constexpr (!in_fixed_point<P, 0>) {
-        nr = newton_in<BLK, false, false>(w, w.at(WS_DL), exp_table(), d.ph.tol, d.ph.min_upd,
-                                          maxit, false);
-      } else if (!d.ph.fx || !newton_fx<BLK, true, false>(w, lam.p, BLK, d.ph, maxit, false, nr, moved)) {
-        targets<BLK>(ux, uy, uz, TT, m);
-        gaussian_guess_out<BLK>(ux, uy, uz, TT, lam);
-        nr = newton<BLK, false>(w, d.ph.tol, d.ph.min_upd, maxit, false);
-      }
-      if (nr.failed) {
-        targets<BLK>(ux, uy, uz, TT, m);
-        fallback_cell<BLK>(d.lam, d.Np, cell, w, TT, false);
-      }
-      store_solver_state<BLK>(d, cell, w);
-      const double cgr = d.ph.cg * TT * rr;
-      for (int i = 0; i < Q; ++i) {
-        pop[(long long)i * d.Np + cell] = to_store<P>(d, i, rr * F[i]);
-        pop[(long long)(Q + i) * d.Np + cell] = to_store<P>(d, Q + i, cgr * F[i]);
-      }
-      atomicAdd(&s_ctr[CTR_FAILED], (unsigned)nr.failed);
-    } else {
-      for (int j = 0; j < 2 * Q; ++j) pop[(long long)j * d.Np + cell] = P(0);
-      for (int k = 0; k < SOLVER_PLANES; ++k) d.lam[k * d.Np + cell] = 0.0;
-    }
-  }
+  bool asym = false, left = false;
+  if (r < len && c0 + r < d.N)
+    left = init_cell<P, BLK, FIXED>(d, rho, u, us, T, c0 + r, r, maxit, WS<BLK>{smem + threadIdx.x},
+                                    s_ctr, asym);
+  if constexpr (FIXED) leave(d, list, r, left);
   if (__syncthreads_or(asym) && threadIdx.x == 0) atomicAdd(d.ctr + CTR_ASYM, 1ull);
+  flush_stats<BLK>(s_ctr, d.ctr);
+}
+
+// The initial condition of the cells of the range left by k_init, or with all of every cell,
+// solved in FP64 (FP64 storage).
+template <int BLK>
+__global__ void __launch_bounds__(BLK, solve_min_blocks(false))
+    k_init_fp64(Desc d, const double* rho, const double* u, long long us, const double* T,
+                long long c0, long long len, int maxit, int list, bool all) {
+  extern __shared__ double smem[];
+  __shared__ unsigned int s_ctr[CTR_N];
+  cudaGridDependencySynchronize();
+  if (blockIdx.x == 0 && threadIdx.x == 0) clear_rest(d, list ^ 1);
+  if (!all && d.ctr[CTR_REST + list] == 0) return;
+  for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
+  load_exp_table();
+  bool any = false;
+  for_rest(d, list, all, min(len, d.N - c0), [&](long long r) {
+    bool asym = false;
+    init_cell<double, BLK, false>(d, rho, u, us, T, c0 + r, r, maxit, WS<BLK>{smem + threadIdx.x},
+                                  s_ctr, asym);
+    any = any || asym;
+  });
+  if (__syncthreads_or(any) && threadIdx.x == 0) atomicAdd(d.ctr + CTR_ASYM, 1ull);
   flush_stats<BLK>(s_ctr, d.ctr);
 }
 
@@ -1103,6 +1217,33 @@ static __global__ void k_sum_partials(const double* partials, int nblocks, doubl
   double s = 0.0;
   for (int b = 0; b < nblocks; ++b) s += partials[b * 5 + k];
   out5[k] = s;
+}
+
+// Blocks of the FP64 kernel of n cells: as many as are resident at a time for the few cells that a
+// fixed-point kernel leaves, else one warp for 32 cells.
+inline unsigned fp64_blocks(long long n, bool all) {
+  const long long blocks = ((n + 31) / 32 + solve_blk(false) / 32 - 1) / (solve_blk(false) / 32);
+  return (unsigned)(all || blocks < 4 * 152 ? blocks : 4 * 152);
+}
+
+// One time step over every fluid cell, without the boundary fills.
+template <class P, bool D2, bool PR, int SOLVER>
+void launch_step(const Desc& d, bool odd, cudaStream_t stream) {
+  constexpr bool FIXED = in_fixed_point<P, SOLVER>;
+  constexpr int BLK = solve_blk(FIXED);
+  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
+  if (!FIXED || d.ph.fx) {
+    if (odd) launch_ws<k_step<true, P, BLK, D2, PR, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
+    else launch_ws<k_step<false, P, BLK, D2, PR, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
+  }
+  const bool all = !d.ph.fx;
+  if constexpr (FIXED) {
+    const unsigned grid64 = fp64_blocks(d.N, all);
+    constexpr int B = solve_blk(false);
+    constexpr size_t WSB = ws_bytes(false);
+    if (odd) launch_ws_early<k_step_fp64<true, D2, PR, SOLVER>>(grid64, B, WSB, stream, d, all);
+    else launch_ws_early<k_step_fp64<false, D2, PR, SOLVER>>(grid64, B, WSB, stream, d, all);
+  }
 }
 
 }  // namespace lbm39

@@ -46,7 +46,7 @@ struct Range {
 };
 
 struct AuxLayout {
-  size_t lam, ctr, heq, href, fstore, partials, result, stage, total;
+  size_t lam, ctr, heq, href, fstore, partials, result, stage, rest, total;
 };
 
 long long plane_stride(long long N) { return (N + 63) / 64 * 64; }
@@ -65,7 +65,11 @@ AuxLayout aux_layout(long long N) {
   a.partials = off; off = align256(off + sizeof(double) * 5 * RED_BLOCKS);
   a.result = off; off = align256(off + sizeof(double) * 8);
   a.stage = off; off = align256(off + sizeof(double) * 6 * std::min(N, STAGE_CELLS));
-  a.total = off;
+  // The list of the cells left to an FP64 kernel, an entry for each 32 cells at most, shares the
+  // sixth staging plane: lbm39_init_host stages five, and a read-out comes before or after a step
+  // on the lattice's stream.  Above 2^25 cells it needs more than that plane.
+  a.rest = a.stage + sizeof(double) * 5 * std::min(N, STAGE_CELLS);
+  a.total = std::max(off, align256(a.rest + sizeof(Rest) * ((N + 31) / 32)));
   return a;
 }
 
@@ -170,41 +174,35 @@ struct Launch {
   static constexpr size_t WSB = ws_bytes(FIXED);
   static void step(lbm39_lattice* L, bool odd) {
     L->desc.t = L->t;
-    const unsigned grid = (unsigned)((L->N + BLK - 1) / BLK);
     const unsigned fgrid = (unsigned)((L->N + 255) / 256);
     // the reduced (z-mirror) system serves the FP64 path only (see reduction_allowed)
     constexpr bool fp64 = sizeof(P) == 8;
-    if (fp64 && L->p.root_finder != 0) {  // other root finders (root_finders.cu)
+    if (fp64 && L->p.root_finder != 0)  // other root finders (root_finders.cu)
       launch_step_root_finder(L->desc, odd, L->p.root_finder, L->stream);
-      if (L->fills) {
-        if (odd) k_fill_odd<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
-        else k_fill_even<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
-      }
-      return;
-    }
-    if (L->desc.ph.pr_adjust) {  // Prandtl-number adjustment (prandtl.cu)
+    else if (L->desc.ph.pr_adjust)  // Prandtl-number adjustment (prandtl.cu)
       launch_step_prandtl(L->desc, odd, !fp64, L->stream);
-      if (L->fills) {
-        if (odd) k_fill_odd<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
-        else k_fill_even<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
-      }
-      return;
-    }
-    if (!odd) {
-      if (fp64 && L->desc.d2) launch_ws<k_step<false, P, BLK, fp64>>(grid, BLK, WSB, L->stream, L->desc);
-      else launch_ws<k_step<false, P, BLK, false>>(grid, BLK, WSB, L->stream, L->desc);
-      if (L->fills) k_fill_even<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
-    } else {
-      if (fp64 && L->desc.d2) launch_ws<k_step<true, P, BLK, fp64>>(grid, BLK, WSB, L->stream, L->desc);
-      else launch_ws<k_step<true, P, BLK, false>>(grid, BLK, WSB, L->stream, L->desc);
-      if (L->fills) k_fill_odd<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
-    }
+    else if (fp64 && L->desc.d2)
+      launch_step<P, fp64, false, 0>(L->desc, odd, L->stream);
+    else
+      launch_step<P, false, false, 0>(L->desc, odd, L->stream);
+    if (!L->fills) return;
+    if (odd) k_fill_odd<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
+    else k_fill_even<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
   }
   static void init(lbm39_lattice* L, const double* rho, const double* u, long long us,
-                   const double* T, long long c0, long long len) {
+                   const double* T, long long c0, long long len, int range) {
+    const int list = 2 + (range & 1);
     const unsigned grid = (unsigned)((len + BLK - 1) / BLK);
-    launch_ws<k_init<P, BLK>>(grid, BLK, WSB, L->stream, L->desc, rho, u, us, T, c0, len,
-                              L->p.init_maxit);
+    const int maxit = L->p.init_maxit;
+    if (!FIXED || L->desc.ph.fx)
+      launch_ws<k_init<P, BLK>>(grid, BLK, WSB, L->stream, L->desc, rho, u, us, T, c0, len, maxit,
+                                list);
+    const bool all = !L->desc.ph.fx;
+    if constexpr (FIXED) {
+      constexpr int B = solve_blk(false);
+      launch_ws_early<k_init_fp64<B>>(fp64_blocks(len, all), B, ws_bytes(false), L->stream, L->desc, rho,
+                                u, us, T, c0, len, maxit, list, all);
+    }
   }
   static void macros(lbm39_lattice* L, double* rho, double* u, long long us, double* T,
                      double* p, long long c0, long long len) {
@@ -357,6 +355,7 @@ int lbm39_create(const lbm39_params* p, const int32_t* vel, const double* w, voi
   Desc& d = L->desc;
   d.pop = pop_buf;
   d.lam = reinterpret_cast<double*>(L->aux + L->lay.lam);
+  d.rest = reinterpret_cast<Rest*>(L->aux + L->lay.rest);
   d.mask = mask_dev;
   d.ctr = L->ctr();
   d.heq_inf = reinterpret_cast<const double*>(L->aux + L->lay.heq);
@@ -454,9 +453,9 @@ static void* mapped_host(const void* p, size_t bytes) {
 }
 
 static int init_range(lbm39_lattice* L, const double* rho, const double* u, long long us,
-                      const double* T, long long c0, long long len) {
-  if (L->mixed) Launch<float>::init(L, rho, u, us, T, c0, len);
-  else Launch<double>::init(L, rho, u, us, T, c0, len);
+                      const double* T, long long c0, long long len, int range = 0) {
+  if (L->mixed) Launch<float>::init(L, rho, u, us, T, c0, len, range);
+  else Launch<double>::init(L, rho, u, us, T, c0, len, range);
   return last_launch();
 }
 
@@ -522,7 +521,7 @@ int lbm39_init_host(lbm39_lattice* L, const double* rho, const double* u, const 
       CUDA_OK(cudaMemcpyAsync(s + (1 + a) * C, u + a * L->N + c0, sizeof(double) * n,
                               cudaMemcpyHostToDevice, L->stream));
     CUDA_OK(cudaMemcpyAsync(s + 4 * C, T + c0, sizeof(double) * n, cudaMemcpyHostToDevice, L->stream));
-    rc = init_range(L, s, s + C, C, s + 4 * C, c0, n);
+    rc = init_range(L, s, s + C, C, s + 4 * C, c0, n, (int)(c0 / C));
     if (rc) return rc;
   }
   return init_end(L);
@@ -798,13 +797,23 @@ BatchLayout batch_layout(int maxlat, long long maxcells) {
 template <class P>
 int batch_enqueue(lbm39_batch* B, int s) {
   const int nt = (int)B->hT.size(), nf = (int)B->hF.size(), n2 = B->nT2;
+  const int nlat = (int)B->hE.size();
   constexpr int BLK = Launch<P>::BLK;
   constexpr size_t WSB = Launch<P>::WSB;
+  constexpr int BLK64 = solve_blk(false);
   if constexpr (sizeof(P) == 8) {
-    if (n2) launch_ws<k_batch_step<P, BLK, true>>(n2, BLK, WSB, B->stream, B->dE, B->dT, s);
+    if (n2) {
+      launch_ws<k_batch_step<P, BLK, true>>(n2, BLK, WSB, B->stream, B->dE, B->dT, s);
+      launch_ws_early<k_batch_step_fp64<true>>(fp64_blocks((long long)n2 * BLK, false), BLK64,
+                                         ws_bytes(false), B->stream, B->dE, nlat, s);
+    }
   }
-  if (nt > n2)
+  if (nt > n2) {
     launch_ws<k_batch_step<P, BLK, false>>(nt - n2, BLK, WSB, B->stream, B->dE, B->dT + n2, s);
+    if constexpr (sizeof(P) == 8)
+      launch_ws_early<k_batch_step_fp64<false>>(fp64_blocks((long long)(nt - n2) * BLK, false), BLK64,
+                                          ws_bytes(false), B->stream, B->dE, nlat, s);
+  }
   if (nf) k_batch_fill<P><<<nf, 256, 0, B->stream>>>(B->dE, B->dF, s);
   return last_launch();
 }

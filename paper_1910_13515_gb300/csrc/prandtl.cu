@@ -12,20 +12,9 @@
 
 namespace lbm39 {
 
-namespace {
-template <class P>
-void launch(const Desc& d, bool odd, cudaStream_t stream) {
-  constexpr bool FIXED = in_fixed_point<P, 0>;
-  constexpr int BLK = solve_blk(FIXED);
-  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
-  if (odd) launch_ws<k_step<true, P, BLK, false, true>>(grid, BLK, ws_bytes(FIXED), stream, d);
-  else launch_ws<k_step<false, P, BLK, false, true>>(grid, BLK, ws_bytes(FIXED), stream, d);
-}
-}  // namespace
-
 bool launch_step_prandtl(const Desc& d, bool odd, bool mixed, cudaStream_t stream) {
-  if (mixed) launch<float>(d, odd, stream);
-  else launch<double>(d, odd, stream);
+  if (mixed) launch_step<float, false, true, 0>(d, odd, stream);
+  else launch_step<double, false, true, 0>(d, odd, stream);
   return cudaGetLastError() == cudaSuccess;
 }
 

@@ -15,16 +15,8 @@ namespace lbm39 {
 namespace {
 template <int SOLVER>
 void launch(const Desc& d, bool odd, cudaStream_t stream) {
-  constexpr bool FIXED = in_fixed_point<double, SOLVER>;
-  constexpr int BLK = solve_blk(FIXED);
-  const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
-  if (d.d2) {
-    if (odd) launch_ws<k_step<true, double, BLK, true, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
-    else launch_ws<k_step<false, double, BLK, true, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
-  } else {
-    if (odd) launch_ws<k_step<true, double, BLK, false, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
-    else launch_ws<k_step<false, double, BLK, false, false, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
-  }
+  if (d.d2) launch_step<double, true, false, SOLVER>(d, odd, stream);
+  else launch_step<double, false, false, SOLVER>(d, odd, stream);
 }
 }  // namespace
 
