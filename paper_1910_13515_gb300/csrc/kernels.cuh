@@ -1145,9 +1145,11 @@ __global__ void k_macros(Desc d, double* rho, double* u, long long us, double* T
 
 // Conserved sums over fluid cells (mass, momentum, total energy): fixed
 // grid-stride assignment and fixed-order tree reductions, so the result is
-// deterministic.  partials: gridDim.x * 5 doubles.
+// deterministic.  partials: gridDim.x * 5 doubles.  Three blocks an SM: the loads wait for memory,
+// and at the 246 registers that the odd gather otherwise takes lbm39_stats of a 64^3 box took 190 us
+// instead of 179.
 template <bool ODD, class P, int BLK>
-__global__ void __launch_bounds__(BLK) k_conserved(Desc d, double* partials) {
+__global__ void __launch_bounds__(BLK, 3) k_conserved(Desc d, double* partials) {
   __shared__ double red[5][BLK];
   double acc[5] = {0, 0, 0, 0, 0};
   for (long long cell = (long long)blockIdx.x * BLK + threadIdx.x; cell < d.N;
