@@ -48,6 +48,7 @@ struct Phys {
   int maxit;        // Newton updates allowed
   int min_upd;      // updates taken even from a converged warm start
   unsigned long long tol_fx, tol_fx100;  // tol and tol/100 in units 2^-58 (the fixed-point solve)
+  int g_shift;      // g_shift(cg)
   int fx;           // the fixed-point solve resolves tol (else every solve is FP64)
   int kn_sensor;    // Eq. (alpha) on/off
   double omega[4];  // 1 / (tau alpha) for the four branches of Eq. (alpha) (1/tau without

@@ -119,6 +119,15 @@ __device__ __forceinline__ u64 unit58(double F, int top = 1023) {
   return m >> s;
 }
 
+// The same for F of either sign, |F| 2^(1023 - top) below 2: rounded down, as a 64-bit integer.
+__device__ __forceinline__ u64 floor58(double F, int top) {
+  const unsigned hi = (unsigned)__double2hiint(F), lo = (unsigned)__double2loint(F);
+  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  const s64 m = (s64)(((u64)__funnelshift_l(lo, mh, 6) << 32) | (lo << 6));
+  const unsigned s = min((unsigned)top - (hi >> 20 & 0x7ffu), 63u);
+  return (u64)(((int)hi < 0 ? -m : m) >> s);
+}
+
 // A double of magnitude below 32 in units 2^-58, rounded toward zero.
 __device__ __forceinline__ s64 signed58(double v) {
   const int h = __double2hiint(v);

@@ -22,6 +22,7 @@
 // A fluid cell's step runs in three phases: gather and moments; targets and
 // Newton (F, lam, m in shared memory); gather again, sensor, BGK and push.
 #pragma once
+#include <cmath>
 #include <cstdint>
 
 #include "cell.cuh"
@@ -169,6 +170,13 @@ __device__ __forceinline__ void push_pair(const Desc& d, long long cell, const N
   if constexpr (D2 && zmirror(i) != i) push<ODD, P, zmirror(i)>(d, cell, nb, base, v);
 }
 
+// The smallest j >= 0 with c_g <= 2.5 2^j: g_i = c_g T f_i divided by 2^j stays in the range that the
+// integer sums give the g_i up to T = 0.8 (in most cells beyond), and at c_g = 2 (gamma = 1.4) has the
+// unit of the f_i.
+inline int g_shift(double cg) {
+  return cg > 2.5 ? std::ilogb(std::nextafter(cg / 2.5, 0.0)) + 1 : 0;
+}
+
 // Raw moments of a cell: rho, j = rho u, e2 = sum f|xi|^2 + sum g = 2 rho E.
 struct Raw {
   double rho, jx, jy, jz, e2;
@@ -220,49 +228,102 @@ __device__ __noinline__ void gather_moments_fp64(const void* pop, long long Np, 
   *M = macro_from_moments(r.rho, r.jx, r.jy, r.jz, r.e2, inv_2cv);
 }
 
-// The macroscopic variables of a cell of a lattice one cell thick in z with the sums formed in
-// 64-bit integers: 158 FP64 additions less, each of which takes the issue time of 60 FP32
-// operations.  D2: of a z-mirror-symmetric one, with one of each mirror pair read (28 % less) and
-// the same values.
-// The populations are scaled by the power of two that brings the largest f_i into [0.25, 0.5) and
-// rounded down to units of 2^-58 (about 2^-56 of the density; the largest are exact); the sums are
-// exact.  Rounding down takes half a unit from each of the 24 populations with |xi_i|^2 >= 4 on
-// average, which is given back.  Where a population is negative, or g or the sums leave the range,
-// the cell's sums are formed in FP64.
+// The sum of the g_i of a cell in units 2^(-58 - kg), with the scale kg at which the largest |g_i| is
+// in [0.25, 0.5), or k if that is smaller; out of line.  False for infinities and NaN, and without
+// SIGNED for negative ones.
+template <bool ODD, bool D2, bool SIGNED>
+__device__ __noinline__ bool g_sum_again(const void* pop, long long Np, long long cell,
+                                         const Nbr* nb, int k, fx::u64* gs, int* kg) {
+  Desc d;
+  d.pop = const_cast<void*>(pop);
+  d.Np = Np;
+  double g[Q];
+  gather<ODD, double, D2>(d, cell, *nb, Q, g);
+  unsigned gmax = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i)
+    gmax = max(gmax, (unsigned)__double2hiint(g[i]) & (SIGNED ? 0x7fffffffu : 0xffffffffu));
+  if (gmax > (2000u << 20)) return false;
+  const int scale = min(1021 - (int)(gmax >> 20), k);
+  fx::u64 sum = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) sum += fx::floor58(g[i], 1023 - scale);
+  *gs = sum;
+  *kg = scale;
+  return true;
+}
+
+// The macroscopic variables of a cell with the sums formed in 64-bit integers, for the lattices one
+// cell thick in z and for the comparison model: 158 FP64 additions less, each of which takes the
+// issue time of 60 FP32 operations.  D2: of a z-mirror-symmetric lattice, with one of each mirror
+// pair read (28 % less) and the same values.
+// The f_i are scaled by the power of two that brings the largest into [0.25, 0.5) and rounded down
+// to units of 2^-58 (about 2^-56 of the density; the largest are exact); the sums are exact.
+// Rounding down takes half a unit from each of the 24 populations with |xi_i|^2 >= 4 on average,
+// which is given back.  The g_i = c_g T f_i have the scale of the f_i divided by the power of two of
+// c_g, and where one of them is beyond it, they are read again with the scale of their largest.
+// SIGNED: with populations of either sign (the comparison model's polynomials, from Ma 0.6 on);
+// where there is a negative one, two bits fewer leave room for the sums.  Else a cell that has one is
+// summed in FP64, as is one whose values or sums leave the ranges.
+// (With FP64 sums for the cells that have negative f_i, or g_i above the scale of the f_i, 20 steps of
+// the comparison model on 1024 x 1024 took 19.6 ms at gamma 1.2 and 19.4 at rms Ma 1; now 14.8, as at
+// gamma 1.4 and Ma 0.3, and 18.6 with FP64 sums for all cells.)
 // On the 1024 x 512 airfoil (few solver updates) a step takes 261 us with these sums and 318 with
-// FP64 ones.  The 3-D lattices keep FP64 sums: their kernel, with the 13-multiplier solve, is bound
-// by instruction fetches, and the longer code took a step of a 128^3 box from 4.2 to 4.5 ms.
+// FP64 ones.  The other 3-D lattices keep FP64 sums: their kernel, with the 13-multiplier solve, is
+// bound by instruction fetches, and the longer code took a step of a 128^3 box from 4.2 to 4.5 ms.
 // f: the gathered f_i, for the caller.
-template <bool ODD, bool D2>
+template <bool ODD, bool D2, bool SIGNED = false>
 __device__ __forceinline__ Macro gather_moments_fx(const Desc& d, long long cell, const Nbr& nb,
                                                    double (&f)[Q]) {
   constexpr int NS = D2 ? 4 : 5;
+  constexpr unsigned ABS = SIGNED ? 0x7fffffffu : 0xffffffffu;
+  const auto units = [](double v, int k) {
+    if constexpr (SIGNED) return fx::floor58(v, 1023 - k);
+    else return fx::unit58(v, 1023 - k);
+  };
   fx::u64 s[NS], gs = 0;
-  unsigned fmax = 0, gmax = 0;
+  unsigned fmax = 0, fneg = 0;
   gather<ODD, double, D2>(d, cell, nb, 0, f);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) fmax = max(fmax, (unsigned)__double2hiint(f[i]));
-  const int k = 1021 - (int)(fmax >> 20);
-  const auto val = [&](auto I) { return fx::unit58(f[decltype(I)::value], 1023 - k); };
+  for (int i = 0; i < Q; ++i) {
+    fmax = max(fmax, (unsigned)__double2hiint(f[i]) & ABS);
+    fneg |= (unsigned)__double2hiint(f[i]);
+  }
+  const bool neg = SIGNED && (int)fneg < 0;
+  // neg: |f_i| < 1/8, so that sum |f_i| |xi_i|^2 <= 204/8 < 32
+  const int k = 1021 - (int)(fmax >> 20) - (neg ? 2 : 0);
+  const auto val = [&](auto I) { return units(f[decltype(I)::value], k); };
   if constexpr (D2) gen::macro_fx2d(val, s);
   else gen::macro_fx(val, s);
+  int kg = k - d.ph.g_shift;
+  bool again, out = false;
   {
     double g[Q];
+    unsigned gmax = 0, gneg = 0;
     gather<ODD, double, D2>(d, cell, nb, Q, g);
     static_for<0, Q>([&](auto I) {
       constexpr int i = decltype(I)::value;
       if constexpr (!D2 || zmirror(i) >= i) {
-        gmax = max(gmax, (unsigned)__double2hiint(g[i]));
-        const fx::u64 u = fx::unit58(g[i], 1023 - k);
+        gmax = max(gmax, (unsigned)__double2hiint(g[i]) & ABS);
+        gneg |= (unsigned)__double2hiint(g[i]);
+        const fx::u64 u = units(g[i], kg);
         gs += D2 && zmirror(i) != i ? 2 * u : u;
       }
     });
+    // beyond the scale (neg: |g_i| < 1/4, else g_i < 1), NaN, or negative on its own
+    again = gmax >= (unsigned)((neg ? 1021 : 1023) - kg) << 20 || (SIGNED && !neg && (int)gneg < 0);
+  }
+  if (again) {
+    const Nbr here = nb;
+    out = !g_sum_again<ODD, D2, SIGNED>(d.pop, d.Np, cell, &here, k, &gs, &kg);
   }
   constexpr int E = NS - 1;
-  // scaled: f_i < 0.5 and sum f < 7, so sum f |xi|^2 < 63; g_i < 1, so sum g < 39
-  if (fmax - (100u << 20) > (1900u << 20) || gmax >= (unsigned)(1023 - k) << 20 ||
-      (unsigned)(s[0] >> 32) > (7u << 26) ||
-      ((unsigned)(s[E] >> 32) >> 1) + ((unsigned)(gs >> 32) >> 1) > (60u << 25)) {
+  // without neg: f_i < 0.5 and sum f < 7, so sum f |xi|^2 < 63; g_i < 1, so sum g < 39.  With neg or
+  // again |sum g| < 20
+  const bool one = !neg && !again && kg == k;  // the energy is one sum
+  if (fmax - (100u << 20) > (1900u << 20) || out ||
+      (!neg && (unsigned)(s[0] >> 32) > (7u << 26)) ||
+      (one && ((unsigned)(s[E] >> 32) >> 1) + ((unsigned)(gs >> 32) >> 1) > (60u << 25))) {
     const Nbr here = nb;
     Macro M;
     gather_moments_fp64<ODD, D2>(d.pop, d.Np, cell, &here, d.ph.inv_2cv, &M);
@@ -271,20 +332,29 @@ __device__ __forceinline__ Macro gather_moments_fx(const Desc& d, long long cell
   // products that are not contracted into the sums that follow: both systems round alike
   const double sc = __hiloint2double((1023 - 58 - k) << 20, 0);
   const auto value = [&](fx::u64 v) { return gen::mul_rn((double)(fx::s64)v, sc); };
-  double jz = 0.0;
+  double jz = 0.0, e2;
   if constexpr (!D2) jz = value(s[3]);
-  return macro_from_moments(value(s[0] + 12), value(s[1]), value(s[2]), jz,
-                            gen::mul_rn((double)(s[E] + gs + 87 + 12), sc), d.ph.inv_2cv);
+  if (one) {
+    e2 = gen::mul_rn((double)(s[E] + gs + 87 + 12), sc);
+  } else {
+    const fx::u64 e = s[E] + 87, g = gs + 12;
+    e2 = gen::mul_rn(neg ? (double)(fx::s64)e : (double)e, sc) +
+         gen::mul_rn(neg || again ? (double)(fx::s64)g : (double)g,
+                     __hiloint2double((1023 - 58 - kg) << 20, 0));
+  }
+  return macro_from_moments(value(s[0] + 12), value(s[1]), value(s[2]), jz, e2, d.ph.inv_2cv);
 }
 
 // The same out of line, for the full system on such lattices.
 template <bool ODD>
 __device__ __noinline__ void gather_moments_thin(const void* pop, long long Np, long long cell,
-                                                 const Nbr* nb, double inv_2cv, Macro* M) {
+                                                 const Nbr* nb, double inv_2cv, int g_shift,
+                                                 Macro* M) {
   Desc d;
   d.pop = const_cast<void*>(pop);
   d.Np = Np;
   d.ph.inv_2cv = inv_2cv;
+  d.ph.g_shift = g_shift;
   double f[Q];
   *M = gather_moments_fx<ODD, false>(d, cell, *nb, f);
 }
@@ -299,7 +369,7 @@ __device__ __forceinline__ Macro step_moments(const Desc& d, long long cell, con
   if (d.nz != 1) return gather_moments<ODD, double>(d, cell, nb);
   const Nbr here = nb;
   Macro M;
-  gather_moments_thin<ODD>(d.pop, d.Np, cell, &here, d.ph.inv_2cv, &M);
+  gather_moments_thin<ODD>(d.pop, d.Np, cell, &here, d.ph.inv_2cv, d.ph.g_shift, &M);
   return M;
 }
 

@@ -369,6 +369,7 @@ int lbm39_create(const lbm39_params* p, const int32_t* vel, const double* w, voi
   d.ph.tau = p->tau;
   d.ph.cg = 2.0 * cv - D;
   d.ph.inv_2cv = 1.0 / (2.0 * cv);
+  d.ph.g_shift = g_shift(d.ph.cg);
   d.ph.tol = p->newton_tol;
   d.ph.maxit = p->newton_maxit;
   d.ph.min_upd = p->newton_min_upd;

@@ -48,10 +48,11 @@ __device__ __forceinline__ double load_pre(const Desc& d, long long cell, const 
 // opp(i) and the odd pass writes over the slot read for opp(i).
 template <bool ODD>
 __device__ __forceinline__ void step_cell(const Desc& d, long long cell) {
-  Nbr nb;
-  if constexpr (ODD) nb = Nbr(d, coord_of(d, cell));
+  Coord c{0, 0, 0};
+  if constexpr (ODD) c = coord_of(d, cell);
   double f[Q];
-  const Macro M = gather_moments_fx<ODD, false>(d, cell, nb, f);
+  const Macro M = gather_moments_fx<ODD, false, true>(d, cell, fresh_nbr<ODD>(d, c), f);
+  const Nbr nb = fresh_nbr<ODD>(d, c);
   const Coef k = coefficients(M.ux * M.ux + M.uy * M.uy + M.uz * M.uz, M.T - TH);
   const double om = d.ph.omega[0];
   const double keep = 1.0 - om;
@@ -177,6 +178,7 @@ int lbm39_poly_create(const lbm39_params* p, void* pop_buf, void* aux_buf, void*
   d.ph.tau = p->tau;
   d.ph.cg = 2.0 * cv - D;
   d.ph.inv_2cv = 1.0 / (2.0 * cv);
+  d.ph.g_shift = g_shift(d.ph.cg);
   for (int b = 0; b < 4; ++b) d.ph.omega[b] = 1.0 / p->tau;
   *out = L;
   return LBM39_OK;
