@@ -91,8 +91,13 @@ typedef struct {
                                u_z and u_inf[2] are all 0, the populations stay mirror
                                symmetric in z, and the FP64 Newton solve uses the nine
                                z-even constraints (the others are exactly zero there):
-                               the same values, less work.  0: always all 13.  The
-                               precision form always solves all 13. */
+                               less work, and the same values wherever both systems
+                               solve.  They can differ in a cell at the edge of the
+                               moment cone: all 13 form z-odd pivots too and may find
+                               one not positive, so that such a cell takes the fallback
+                               (see lbm39_step) or, out of fixed point, an FP64 solve.
+                               0: always all 13.  The precision form always solves all
+                               13. */
   double prandtl;           /* Prandtl number (Sec. 3 leaves its adjustment out: Pr = 1).
                                1 (default) or 0: the paper's BGK collision.  Otherwise a
                                quasi-equilibrium collision with two relaxation times: f

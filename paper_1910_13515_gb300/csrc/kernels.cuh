@@ -708,7 +708,7 @@ __device__ __forceinline__ bool solve_cell(const Desc& d, long long cell, WS<BLK
 // One fluid cell's time step (even or odd AA pass): phases A, B and C, with
 // the Newton statistics added to the block's counters.  w: the cell's workspace.
 // D2: the nine-function constraint system of a z-mirror-symmetric lattice one
-// cell thick in z (Sys<true>; the same values as the full system).
+// cell thick in z (Sys<true>; the same values as the full system wherever both solve).
 // SOLVER: the root finder of the constraint equations (solve_cell).
 // FIXED: solved in fixed point; true, with nothing done, for a cell that is left
 // to the FP64 step.
