@@ -906,7 +906,13 @@ def main():
                   + (model[2] * shares["start32_solve_share"] if len(model) > 2 else 0.0)
                   if model else None)
     achieved_tf = flops_cell * fluid / (step_ms * 1e-3) / 1e12 if model else None
-    hbm_gbs = BYTES_PER_UPDATE[args.precision] * fluid / (step_ms * 1e-3) / 1e9
+    bytes_upd = BYTES_PER_UPDATE[args.precision]
+    if reduced and args.root_finder != "chord":
+        # one of each mirror pair (28 of 39) is read, of the populations and of the stored F, and
+        # the mark; the multipliers are read and the state written back where an update is taken
+        bytes_upd = (2 * 28 + 2 * 39 + 28 + 1) * 8 + (13 + 52) * 8 * (
+            1.0 - shares["newton_updates_share_0_1_2_3_4plus"][0])
+    hbm_gbs = bytes_upd * fluid / (step_ms * 1e-3) / 1e9
     traffic = issue = None
     if (NCU_LAUNCH["kernel_hash"] == kernel_source_hash() and args.mach == 0.8
             and args.root_finder == "newton" and args.newton_tol == 1e-12
@@ -927,7 +933,7 @@ def main():
                                 "DADD/DMUL)") if model else "none fitted for this solver",
                 "hbm": {"achieved_gbs": round(hbm_gbs, 1), "peak_gbs": HBM_PEAK_GBS,
                         "frac": round(hbm_gbs / HBM_PEAK_GBS, 4),
-                        "bytes_per_update": BYTES_PER_UPDATE[args.precision],
+                        "bytes_per_update": round(bytes_upd, 1),
                         "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)"}}
 
     if args.precision == "fp64" and args.root_finder != "chord":

@@ -211,9 +211,9 @@ __device__ __forceinline__ Raw gather_raw(const Desc& d, long long cell, const N
   return r;
 }
 
-template <bool ODD, class P, bool D2 = false>
+template <bool ODD, class P>
 __device__ __forceinline__ Macro gather_moments(const Desc& d, long long cell, const Nbr& nb) {
-  const Raw r = gather_raw<ODD, P, D2>(d, cell, nb);
+  const Raw r = gather_raw<ODD, P>(d, cell, nb);
   return macro_from_moments(r.rho, r.jx, r.jy, r.jz, r.e2, d.ph.inv_2cv);
 }
 
@@ -684,12 +684,14 @@ __device__ __forceinline__ bool solve_cell(const Desc& d, long long cell, WS<BLK
   n32 = 0;
   moved = true;
   bool cached = true;
+  [[maybe_unused]] const unsigned lanes = __activemask();
   if constexpr (START) {
     if (FIXED) load_multipliers<BLK>(d, cell, w);
     if (maxit > 0) {  // a cell on the fallback off a retry step takes no step at all
       n32 = start32<BLK, D2>(w);
       cached = n32 == 0;
     }
+    if constexpr (FIXED) __syncwarp(lanes);  // see step_cell
   }
   if constexpr (FIXED) {
     const double* src = START ? w.p + WS_LAM * BLK : d.lam + cell;
@@ -748,8 +750,9 @@ __device__ __forceinline__ bool step_cell(const Desc& d, long long cell, WS<BLK>
   const bool solved = solve_cell<P, BLK, D2, SOLVER, FIXED>(d, cell, w, maxit, nr, n32, moved);
   if constexpr (FIXED) {
     // the lanes go on together: with the return below, the compiler otherwise left a warp as its
-    // solves had diverged, and phase C ran 1.7 times for each (a 128^3 box 54 ms, not 44.5)
-    __syncwarp(lanes);
+    // solves had diverged, and phase C ran 1.7 times for each (a 128^3 box 54 ms, not 44.5).  With
+    // root finder 3 they come together after its start, where that matters more (2 % on boxes)
+    if constexpr (SOLVER != 3) __syncwarp(lanes);
     if (!solved) return true;
   }
   if (nr.failed) {
@@ -994,9 +997,10 @@ __device__ __forceinline__ P reversed(const Desc& d, P v, int from, int to) {
 // The fill functions take their 39 directions in batches: the masks of a batch, then its
 // populations, are read before the first is stored, and the neighbours are computed where the
 // table of them would lie in local memory.  Few cells have work, and each waits for memory: what
-// counts is that many blocks are resident (40 registers, six blocks of 256) and that a cell waits
-// less often.  On the 1024 x 512 airfoil a fill takes 16 us (even) and 24 us (odd) where the
-// direction-by-direction loops took 40 and 30; batches of 13 took 19 and 37 (128 registers).
+// counts is that many blocks are resident (40 registers, six blocks of 256, with about 250 bytes of
+// spills) and that a cell waits less often.  On the 1024 x 512 airfoil a fill takes 16 us (even) and
+// 24 us (odd) where the direction-by-direction loops took 40 and 30; batches of 13 took 19 and 37
+// (128 registers).
 constexpr int FILL_BATCH = 3;
 static_assert(Q % FILL_BATCH == 0, "whole batches");
 

@@ -22,7 +22,8 @@ namespace poly {
 
 // Threads per block of the cell kernels, and blocks an SM (168 registers): FP64 issue bounds the
 // step (two thirds of the FP64 operations of FP64 sums are left).  40 steps on 2048 x 2048 take
-// 115 ms; with 254 registers 127, with blocks of 128 threads 131, with FP64 sums 151.
+// 113 ms; before the odd pass built its neighbour table twice 115, with 254 registers then 127, with
+// blocks of 128 threads 131, with FP64 sums 151.
 constexpr int BLK = 64, MIN_BLOCKS = 6;
 constexpr int RED_BLOCKS = 1024;  // blocks of the conserved-sum reduction
 constexpr int RED_THREADS = 128;

@@ -15,8 +15,8 @@
 // instructions, and code that grows by a few thousand instructions costs more than
 // it saves; two blocks an SM at 255 registers without spills, and blocks of 64, 192,
 // 256 and 384 threads, with and without a barrier in each iteration, measured 2 to
-// 15 % slower).  On the 128^3 box at rms Ma 0.5 ten steps with the initialisation take 50.0 ms where the
-// FP64 solve took 259.4, on the 256^3 box at rms Ma 0.8 five take 243 where it took 1145.
+// 15 % slower).  On the 128^3 box at rms Ma 0.5 ten steps with the initialisation take 44.5 ms where the
+// FP64 solve took 259.4, on the 256^3 box at rms Ma 0.8 five take 213 where it took 1137.
 #pragma once
 #include "cell.cuh"
 #include "fixed.cuh"
