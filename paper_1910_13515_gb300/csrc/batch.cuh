@@ -56,9 +56,9 @@ __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, 0>)) k
 // The cells that k_batch_step left to the FP64 solve, over the lists of the lattices of its
 // constraint system that have not reached their end time.
 template <bool D2>
-__global__ void __launch_bounds__(solve_blk(false), solve_min_blocks(false))
+__global__ void __launch_bounds__(FP64_BLK, 1)
     k_batch_step_fp64(const BatchEntry* __restrict__ E, int nlat, int s) {
-  constexpr int BLK = solve_blk(false);
+  constexpr int BLK = FP64_BLK;
   extern __shared__ double smem[];
   __shared__ unsigned int s_ctr[BLK / 32][CTR_N];  // a warp's, for one lattice at a time
   __shared__ Desc s_desc[BLK / 32];
@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(solve_blk(false), solve_min_blocks(false))
   load_exp_table();
   cudaGridDependencySynchronize();
   const long long warps = (long long)gridDim.x * (BLK / 32);
-  long long next = (long long)blockIdx.x * (BLK / 32) + warp;  // this warp's next entry
-  long long base = 0;                                          // entries of the lattices before j0
+  long long next = first_entry();  // this warp's next entry
+  long long base = 0;              // entries of the lattices before j0
   for (int j0 = 0; j0 < nlat; j0 += 32) {
     const int j = j0 + lane;
     long long n = 0;

@@ -22,6 +22,7 @@
 // A fluid cell's step runs in three phases: gather and moments; targets and
 // Newton (F, lam, m in shared memory); gather again, sensor, BGK and push.
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -229,9 +230,8 @@ __device__ __noinline__ void gather_moments_fp64(const void* pop, long long Np, 
 }
 
 // The sum of the g_i of a cell in units 2^(-58 - kg), with the scale kg at which the largest |g_i| is
-// in [0.25, 0.5), or k if that is smaller; out of line.  False for infinities and NaN, and without
-// SIGNED for negative ones.
-template <bool ODD, bool D2, bool SIGNED>
+// in [0.25, 0.5), or k if that is smaller; out of line.  False for infinities and NaN.
+template <bool ODD, bool D2>
 __device__ __noinline__ bool g_sum_again(const void* pop, long long Np, long long cell,
                                          const Nbr* nb, int k, fx::u64* gs, int* kg) {
   Desc d;
@@ -242,7 +242,7 @@ __device__ __noinline__ bool g_sum_again(const void* pop, long long Np, long lon
   unsigned gmax = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i)
-    gmax = max(gmax, (unsigned)__double2hiint(g[i]) & (SIGNED ? 0x7fffffffu : 0xffffffffu));
+    gmax = max(gmax, (unsigned)__double2hiint(g[i]) & 0x7fffffffu);
   if (gmax > (2000u << 20)) return false;
   const int scale = min(1021 - (int)(gmax >> 20), k);
   fx::u64 sum = 0;
@@ -261,10 +261,11 @@ __device__ __noinline__ bool g_sum_again(const void* pop, long long Np, long lon
 // to units of 2^-58 (about 2^-56 of the density; the largest are exact); the sums are exact.
 // Rounding down takes half a unit from each of the 24 populations with |xi_i|^2 >= 4 on average,
 // which is given back.  The g_i = c_g T f_i have the scale of the f_i divided by the power of two of
-// c_g, and where one of them is beyond it, they are read again with the scale of their largest.
-// SIGNED: with populations of either sign (the comparison model's polynomials, from Ma 0.6 on);
-// where there is a negative one, two bits fewer leave room for the sums.  Else a cell that has one is
-// summed in FP64, as is one whose values or sums leave the ranges.
+// c_g.  SIGNED (the comparison model): with populations of either sign, which its polynomials give
+// from Ma 0.6 on; where there is a negative one, two bits fewer leave room for the sums; and where a
+// g_i is beyond the scale, the g_i are read again with that of their largest.  Else such a cell is
+// summed in FP64 (the reduced kernel grew by 1.5 % in time with the second reading), as is one whose
+// sums leave the ranges.
 // (With FP64 sums for the cells that have negative f_i, or g_i above the scale of the f_i, 20 steps of
 // the comparison model on 1024 x 1024 took 19.6 ms at gamma 1.2 and 19.4 at rms Ma 1; now 14.8, as at
 // gamma 1.4 and Ma 0.3, and 18.6 with FP64 sums for all cells.)
@@ -313,9 +314,13 @@ __device__ __forceinline__ Macro gather_moments_fx(const Desc& d, long long cell
     // beyond the scale (neg: |g_i| < 1/4, else g_i < 1), NaN, or negative on its own
     again = gmax >= (unsigned)((neg ? 1021 : 1023) - kg) << 20 || (SIGNED && !neg && (int)gneg < 0);
   }
-  if (again) {
-    const Nbr here = nb;
-    out = !g_sum_again<ODD, D2, SIGNED>(d.pop, d.Np, cell, &here, k, &gs, &kg);
+  if constexpr (SIGNED) {
+    if (again) {
+      const Nbr here = nb;
+      out = !g_sum_again<ODD, D2>(d.pop, d.Np, cell, &here, k, &gs, &kg);
+    }
+  } else {
+    out = again;
   }
   constexpr int E = NS - 1;
   // without neg: f_i < 0.5 and sum f < 7, so sum f |xi|^2 < 63; g_i < 1, so sum g < 39.  With neg or
@@ -656,6 +661,10 @@ constexpr bool in_fixed_point = sizeof(P) == 8 && SOLVER != 1;
 // direction there too).
 constexpr int solve_blk(bool fixed) { return fixed ? 128 : 64; }
 constexpr int solve_min_blocks(bool fixed) { return fixed ? 3 : 4; }
+// The FP64 kernels beside the fixed-point ones: one block an SM, as many warps as four blocks of 64
+// (a step's launch that finds nothing to do is over sooner with 152 blocks than with 608).
+constexpr int FP64_BLK = 256;
+constexpr size_t FP64_WS_BYTES = (size_t)FP64_BLK * WS_DOUBLES * sizeof(double);
 constexpr size_t ws_bytes(bool fixed) {
   return (size_t)solve_blk(fixed) * (fixed ? WS_DOUBLES_FX : WS_DOUBLES) * sizeof(double);
 }
@@ -799,19 +808,24 @@ __device__ __forceinline__ long long next_entry(unsigned long long* taken, long 
   return warps + (long long)__shfl_sync(0xffffffffu, e, 0);
 }
 
+// This warp's first entry: neighbouring entries go to different SMs.
+__device__ __forceinline__ long long first_entry() {
+  return (long long)(threadIdx.x / 32) * gridDim.x + blockIdx.x;
+}
+
 // Calls f(cell) for each cell of list k, or with all for each of n cells; a warp takes the 32 cells
 // of an entry together, as the fixed-point kernel had them.
 template <class F>
 __device__ __forceinline__ void for_rest(const Desc& d, int k, bool all, long long n, F&& f) {
   const long long warps = (long long)gridDim.x * (blockDim.x / 32);
   const long long count = all ? (n + 31) / 32 : (long long)d.ctr[CTR_REST + k];
-  long long e = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  long long e = first_entry();
   while (e < count) {
     const Rest r = all ? Rest{(unsigned)e, 0xffffffffu} : d.rest[e];
     const long long cell = (long long)r.w * 32 + (threadIdx.x & 31);
     if ((r.bits >> (threadIdx.x & 31) & 1) && cell < n) f(cell);
     __syncwarp();
-    e = all ? count : next_entry(d.ctr + CTR_TAKEN + k, warps);
+    e = next_entry(d.ctr + CTR_TAKEN + k, warps);
   }
 }
 
@@ -828,6 +842,7 @@ __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, SOLVER
   __shared__ unsigned int s_ctr[CTR_N];
   for (int k = threadIdx.x; k < CTR_N; k += BLK) s_ctr[k] = 0;
   load_solver_table<in_fixed_point<P, SOLVER>>();
+  cudaGridDependencySynchronize();  // launch_step
   const long long cell = (long long)blockIdx.x * BLK + threadIdx.x;
   bool left = false;
   if (cell < d.N && (d.mask == nullptr || d.mask[cell] == MASK_FLUID))
@@ -840,9 +855,8 @@ __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, SOLVER
 // lattices whose tolerance is below the fixed-point resolution (at 1e-13 a 64^3 box's 8 steps take
 // 24.6 ms; 25.4 where the fixed-point kernel called the FP64 solve for each cell).
 template <bool ODD, bool D2, bool PR, int SOLVER>
-__global__ void __launch_bounds__(solve_blk(false), solve_min_blocks(false))
-    k_step_fp64(Desc d, bool all) {
-  constexpr int BLK = solve_blk(false);
+__global__ void __launch_bounds__(FP64_BLK, 1) k_step_fp64(Desc d, bool all) {
+  constexpr int BLK = FP64_BLK;
   extern __shared__ double smem[];
   __shared__ unsigned int s_ctr[CTR_N];
   cudaGridDependencySynchronize();
@@ -940,7 +954,7 @@ __global__ void __launch_bounds__(BLK, solve_min_blocks(in_fixed_point<P, 0>)) k
 // The initial condition of the cells of the range left by k_init, or with all of every cell,
 // solved in FP64 (FP64 storage).
 template <int BLK>
-__global__ void __launch_bounds__(BLK, solve_min_blocks(false))
+__global__ void __launch_bounds__(BLK, 1)
     k_init_fp64(Desc d, const double* rho, const double* u, long long us, const double* T,
                 long long c0, long long len, int maxit, int list, bool all) {
   extern __shared__ double smem[];
@@ -1295,11 +1309,9 @@ static __global__ void k_sum_partials(const double* partials, int nblocks, doubl
   out5[k] = s;
 }
 
-// Blocks of the FP64 kernel of n cells: as many as are resident at a time for the few cells that a
-// fixed-point kernel leaves, else one warp for 32 cells.
-inline unsigned fp64_blocks(long long n, bool all) {
-  const long long blocks = ((n + 31) / 32 + solve_blk(false) / 32 - 1) / (solve_blk(false) / 32);
-  return (unsigned)(all || blocks < 4 * 152 ? blocks : 4 * 152);
+// Blocks of the FP64 kernel of n cells: one an SM, or a warp for each 32 cells.
+inline unsigned fp64_blocks(long long n) {
+  return (unsigned)std::min((n + 31) / 32, 152LL);
 }
 
 // One time step over every fluid cell, without the boundary fills.
@@ -1309,14 +1321,24 @@ void launch_step(const Desc& d, bool odd, cudaStream_t stream) {
   constexpr int BLK = solve_blk(FIXED);
   const unsigned grid = (unsigned)((d.N + BLK - 1) / BLK);
   if (!FIXED || d.ph.fx) {
-    if (odd) launch_ws<k_step<true, P, BLK, D2, PR, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
-    else launch_ws<k_step<false, P, BLK, D2, PR, SOLVER>>(grid, BLK, ws_bytes(FIXED), stream, d);
+    // where all blocks are resident at once the set-up is worth hiding; with more waves the blocks
+    // set up early land unevenly on the SMs (shear layers of 300^2 and 330^2 took 4 and 5 % longer)
+    constexpr size_t WSB = ws_bytes(FIXED);
+    constexpr auto even = k_step<false, P, BLK, D2, PR, SOLVER>;
+    constexpr auto odd_ = k_step<true, P, BLK, D2, PR, SOLVER>;
+    if (grid <= 152u * solve_min_blocks(FIXED)) {
+      if (odd) launch_ws_early<odd_>(grid, BLK, WSB, stream, d);
+      else launch_ws_early<even>(grid, BLK, WSB, stream, d);
+    } else {
+      if (odd) launch_ws<odd_>(grid, BLK, WSB, stream, d);
+      else launch_ws<even>(grid, BLK, WSB, stream, d);
+    }
   }
   const bool all = !d.ph.fx;
   if constexpr (FIXED) {
-    const unsigned grid64 = fp64_blocks(d.N, all);
-    constexpr int B = solve_blk(false);
-    constexpr size_t WSB = ws_bytes(false);
+    const unsigned grid64 = fp64_blocks(d.N);
+    constexpr int B = FP64_BLK;
+    constexpr size_t WSB = FP64_WS_BYTES;
     if (odd) launch_ws_early<k_step_fp64<true, D2, PR, SOLVER>>(grid64, B, WSB, stream, d, all);
     else launch_ws_early<k_step_fp64<false, D2, PR, SOLVER>>(grid64, B, WSB, stream, d, all);
   }

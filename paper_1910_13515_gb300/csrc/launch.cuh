@@ -31,9 +31,10 @@ void launch_ws(unsigned grid, int blk, size_t bytes, cudaStream_t stream, Args..
   Kernel<<<grid, blk, bytes, stream>>>(args...);
 }
 
-// The same for a kernel that begins with cudaGridDependencySynchronize: its blocks are set up while
-// the kernel before it on the stream ends.  For the launches that mostly find nothing to do (2.5 us
-// between two steps of a small lattice, 4.5 us launched as usual).
+// The same for a kernel that calls cudaGridDependencySynchronize before it touches what another has
+// written: its blocks are set up while the kernel before it on the stream ends.  With the step's two
+// kernels launched so, 20 steps of a 105 x 105 lattice take 0.91 ms; with only the second 0.96, and
+// 0.92 where the step was one kernel.
 template <auto Kernel, class... Args>
 void launch_ws_early(unsigned grid, int blk, size_t bytes, cudaStream_t stream, Args... args) {
   allow_shared<Kernel>(bytes);

@@ -190,19 +190,22 @@ struct Launch {
     else k_fill_even<P><<<fgrid, 256, 0, L->stream>>>(L->desc);
   }
   static void init(lbm39_lattice* L, const double* rho, const double* u, long long us,
-                   const double* T, long long c0, long long len, int range) {
-    const int list = 2 + (range & 1);
+                   const double* T, long long c0, long long len, int list) {
     const unsigned grid = (unsigned)((len + BLK - 1) / BLK);
-    const int maxit = L->p.init_maxit;
-    if (!FIXED || L->desc.ph.fx)
-      launch_ws<k_init<P, BLK>>(grid, BLK, WSB, L->stream, L->desc, rho, u, us, T, c0, len, maxit,
-                                list);
-    const bool all = !L->desc.ph.fx;
-    if constexpr (FIXED) {
-      constexpr int B = solve_blk(false);
-      launch_ws_early<k_init_fp64<B>>(fp64_blocks(len, all), B, ws_bytes(false), L->stream, L->desc, rho,
-                                u, us, T, c0, len, maxit, list, all);
+    if (FIXED && !L->desc.ph.fx) {
+      init_fp64(L, rho, u, us, T, c0, len, list, true);
+      return;
     }
+    launch_ws<k_init<P, BLK>>(grid, BLK, WSB, L->stream, L->desc, rho, u, us, T, c0, len,
+                              L->p.init_maxit, list);
+  }
+  // What the fixed-point kernel left of the range, or with all the whole range.
+  static void init_fp64(lbm39_lattice* L, const double* rho, const double* u, long long us,
+                        const double* T, long long c0, long long len, int list, bool all) {
+    constexpr int B = FP64_BLK;
+    if constexpr (FIXED)
+      launch_ws_early<k_init_fp64<B>>(fp64_blocks(len), B, FP64_WS_BYTES, L->stream, L->desc, rho,
+                                      u, us, T, c0, len, L->p.init_maxit, list, all);
   }
   static void macros(lbm39_lattice* L, double* rho, double* u, long long us, double* T,
                      double* p, long long c0, long long len) {
@@ -454,11 +457,13 @@ static void* mapped_host(const void* p, size_t bytes) {
 }
 
 static int init_range(lbm39_lattice* L, const double* rho, const double* u, long long us,
-                      const double* T, long long c0, long long len, int range = 0) {
-  if (L->mixed) Launch<float>::init(L, rho, u, us, T, c0, len, range);
-  else Launch<double>::init(L, rho, u, us, T, c0, len, range);
+                      const double* T, long long c0, long long len, int list) {
+  if (L->mixed) Launch<float>::init(L, rho, u, us, T, c0, len, list);
+  else Launch<double>::init(L, rho, u, us, T, c0, len, list);
   return last_launch();
 }
+
+constexpr int INIT_LIST = 2;  // the lists 2 and 3 are those of alternate ranges
 
 static int init_begin(lbm39_lattice* L) {
   CUDA_OK(cudaMemsetAsync(L->pop, 0, L->pop_bytes(), L->stream));
@@ -481,13 +486,29 @@ static bool reduction_allowed(const lbm39_lattice* L) {
          !L->desc.ph.pr_adjust;
 }
 
-// After the init kernels: waits for them and fixes the constraint system.
-static int init_end(lbm39_lattice* L) {
-  unsigned long long asym = 0;
-  CUDA_OK(cudaMemcpyAsync(&asym, L->ctr() + CTR_ASYM, sizeof asym, cudaMemcpyDeviceToHost,
-                          L->stream));
+// After the init kernels: waits for them and fixes the constraint system.  *left: the length of the
+// first range's list.
+static int init_end(lbm39_lattice* L, unsigned long long* left = nullptr) {
+  unsigned long long c[CTR_REST + INIT_LIST + 1 - CTR_ASYM];
+  CUDA_OK(cudaMemcpyAsync(c, L->ctr() + CTR_ASYM, sizeof c, cudaMemcpyDeviceToHost, L->stream));
   CUDA_OK(cudaStreamSynchronize(L->stream));
-  L->desc.d2 = reduction_allowed(L) && asym == 0 ? 1 : 0;
+  L->desc.d2 = reduction_allowed(L) && c[0] == 0 ? 1 : 0;
+  if (left) *left = c[CTR_REST + INIT_LIST - CTR_ASYM];
+  return LBM39_OK;
+}
+
+// The initialisation of the whole lattice as one range; the FP64 kernel for what the fixed-point one
+// left is launched where there is such a cell.
+static int init_whole(lbm39_lattice* L, const double* rho, const double* u, const double* T) {
+  int rc = init_range(L, rho, u, L->N, T, 0, L->N, INIT_LIST);
+  if (rc) return rc;
+  unsigned long long left = 0;
+  rc = init_end(L, &left);
+  if (rc || L->mixed || left == 0) return rc;
+  Launch<double>::init_fp64(L, rho, u, L->N, T, 0, L->N, INIT_LIST, false);
+  rc = last_launch();
+  if (rc) return rc;
+  CUDA_OK(cudaStreamSynchronize(L->stream));
   return LBM39_OK;
 }
 
@@ -496,9 +517,7 @@ int lbm39_init(lbm39_lattice* L, const double* rho, const double* u, const doubl
   if (!L || !rho || !u || !T) return LBM39_ERR_ARG;
   int rc = init_begin(L);
   if (rc) return rc;
-  rc = init_range(L, rho, u, L->N, T, 0, L->N);
-  if (rc) return rc;
-  return init_end(L);
+  return init_whole(L, rho, u, T);
 }
 
 int lbm39_init_host(lbm39_lattice* L, const double* rho, const double* u, const double* T) {
@@ -510,12 +529,9 @@ int lbm39_init_host(lbm39_lattice* L, const double* rho, const double* u, const 
   const void* drho = mapped_host(rho, nb);
   const void* du = mapped_host(u, 3 * nb);
   const void* dT = mapped_host(T, nb);
-  if (drho && du && dT) {  // page-locked: the init kernel reads them directly
-    rc = init_range(L, static_cast<const double*>(drho), static_cast<const double*>(du), L->N,
-                    static_cast<const double*>(dT), 0, L->N);
-    if (rc) return rc;
-    return init_end(L);
-  }
+  if (drho && du && dT)  // page-locked: the init kernels read them directly
+    return init_whole(L, static_cast<const double*>(drho), static_cast<const double*>(du),
+                      static_cast<const double*>(dT));
   const long long C = std::min(L->N, STAGE_CELLS);
   double* s = L->stage();
   for (long long c0 = 0; c0 < L->N; c0 += C) {
@@ -525,8 +541,15 @@ int lbm39_init_host(lbm39_lattice* L, const double* rho, const double* u, const 
       CUDA_OK(cudaMemcpyAsync(s + (1 + a) * C, u + a * L->N + c0, sizeof(double) * n,
                               cudaMemcpyHostToDevice, L->stream));
     CUDA_OK(cudaMemcpyAsync(s + 4 * C, T + c0, sizeof(double) * n, cudaMemcpyHostToDevice, L->stream));
-    rc = init_range(L, s, s + C, C, s + 4 * C, c0, n, (int)(c0 / C));
+    if (C == L->N) return init_whole(L, s, s + C, s + 4 * C);
+    const int list = INIT_LIST + (int)(c0 / C & 1);
+    rc = init_range(L, s, s + C, C, s + 4 * C, c0, n, list);
     if (rc) return rc;
+    if (!L->mixed && L->desc.ph.fx) {
+      Launch<double>::init_fp64(L, s, s + C, C, s + 4 * C, c0, n, list, false);
+      rc = last_launch();
+      if (rc) return rc;
+    }
   }
   return init_end(L);
 }
@@ -804,19 +827,18 @@ int batch_enqueue(lbm39_batch* B, int s) {
   const int nlat = (int)B->hE.size();
   constexpr int BLK = Launch<P>::BLK;
   constexpr size_t WSB = Launch<P>::WSB;
-  constexpr int BLK64 = solve_blk(false);
   if constexpr (sizeof(P) == 8) {
     if (n2) {
       launch_ws<k_batch_step<P, BLK, true>>(n2, BLK, WSB, B->stream, B->dE, B->dT, s);
-      launch_ws_early<k_batch_step_fp64<true>>(fp64_blocks((long long)n2 * BLK, false), BLK64,
-                                         ws_bytes(false), B->stream, B->dE, nlat, s);
+      launch_ws_early<k_batch_step_fp64<true>>(fp64_blocks((long long)n2 * BLK), FP64_BLK,
+                                               FP64_WS_BYTES, B->stream, B->dE, nlat, s);
     }
   }
   if (nt > n2) {
     launch_ws<k_batch_step<P, BLK, false>>(nt - n2, BLK, WSB, B->stream, B->dE, B->dT + n2, s);
     if constexpr (sizeof(P) == 8)
-      launch_ws_early<k_batch_step_fp64<false>>(fp64_blocks((long long)(nt - n2) * BLK, false), BLK64,
-                                          ws_bytes(false), B->stream, B->dE, nlat, s);
+      launch_ws_early<k_batch_step_fp64<false>>(fp64_blocks((long long)(nt - n2) * BLK), FP64_BLK,
+                                                FP64_WS_BYTES, B->stream, B->dE, nlat, s);
   }
   if (nf) k_batch_fill<P><<<nf, 256, 0, B->stream>>>(B->dE, B->dF, s);
   return last_launch();
@@ -854,7 +876,9 @@ int lbm39_batch_create(int32_t max_lattices, int64_t max_cells, int32_t precisio
             ? allow_shared<k_batch_step<float, Launch<float>::BLK, false>>(Launch<float>::WSB)
             : allow_shared<k_batch_step<double, Launch<double>::BLK, true>>(Launch<double>::WSB) &&
                   allow_shared<k_batch_step<double, Launch<double>::BLK, false>>(
-                      Launch<double>::WSB)))
+                      Launch<double>::WSB) &&
+                  allow_shared<k_batch_step_fp64<true>>(FP64_WS_BYTES) &&
+                  allow_shared<k_batch_step_fp64<false>>(FP64_WS_BYTES)))
     return LBM39_ERR_CUDA;
   lbm39_batch* B = new (std::nothrow) lbm39_batch;
   if (!B) return LBM39_ERR_ARG;
