@@ -85,10 +85,10 @@ FP64_FLOPS_MODEL = {
 # (profiles/k_step_fixed_point.md has the captures).  The 256^3 figures are the 128^3 captures
 # scaled by the cell count (x 8; the same per-cell work, both far beyond L2; a warp takes the
 # updates of its slowest cell, so the count hardly depends on the mean of its cells).
-NCU_LAUNCH = {"kernel_hash": "f4c0d3664027b73e",
-              "gb": {"box128/fp64": 6.77, "box256/fp64": 54.2, "naca/fp64": 2.88},
-              "warp_instructions": {"box128/fp64": 2.416e9, "box256/fp64": 19.33e9,
-                                    "naca/fp64": 0.3237e9}}
+NCU_LAUNCH = {"kernel_hash": "3a272f277c6418d0",
+              "gb": {"box128/fp64": 6.77, "box256/fp64": 54.1, "naca/fp64": 2.84},
+              "warp_instructions": {"box128/fp64": 2.400e9, "box256/fp64": 19.20e9,
+                                    "naca/fp64": 0.3302e9}}
 # The sources the step kernels and their launches are built from (the serving-form kernels
 # in batch.cuh are not among them).
 KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
@@ -97,9 +97,9 @@ KERNEL_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.c
 # launch (per lattice side n of the n x n x 1 workload; null once the code differs).
 POLY_SOURCES = ("cell.cuh", "d3q39.cuh", "d3q39_gen.cuh", "expd.cuh", "fixed.cuh",
                 "kernels.cuh", "plane.cuh", "solve_fx.cuh", "poly_eq.cuh", "poly.cu")
-POLY_NCU_TRAFFIC = {"kernel_hash": "6e164d1b83de7ee2",
-                    # 2048: mean of an even (5.22) and an odd launch (8.04: it spills)
-                    "gb_per_launch": {"2048": 6.63}}
+POLY_NCU_TRAFFIC = {"kernel_hash": "b949fc4731d2672e",
+                    # 2048: mean of an even (5.25) and an odd launch (5.72)
+                    "gb_per_launch": {"2048": 5.48}}
 
 
 def source_code_text(text: str) -> str:
